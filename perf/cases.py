@@ -219,12 +219,12 @@ def _powers(w, n, q):
 
 def _dft(x, w, q):
     """X_s = sum_j x_j w^(js) mod q over the last axis."""
-    n = x.shape[-1]
-    if n == 1:
-        return x
-    e, o = _dft(x[..., 0::2], w * w % q, q), _dft(x[..., 1::2], w * w % q, q)
-    o = o * _powers(w, n // 2, q) % q
-    return torch.cat([(e + o) % q, (e - o) % q], dim=-1)
+    y = x.unsqueeze(-1)   # [..., r, s]: the transform of the terms j = r (mod the extent of r)
+    while y.shape[-2] > 1:
+        h, m = y.shape[-2] // 2, y.shape[-1]
+        e, o = y[..., :h, :], y[..., h:, :] * _powers(pow(w, h, q), m, q) % q
+        y = torch.cat([(e + o) % q, (e - o) % q], dim=-1)
+    return y[..., 0, :]
 
 
 def _ntt(x, q):
