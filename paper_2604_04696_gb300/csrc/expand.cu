@@ -20,15 +20,25 @@
 // GPU mapping: stage-level kernels (Sec. 4.1.2), one launch per stage, the
 // cluster shape chosen per stage (Sec. 4.4):
 //   - expand_stage_kernel: one thread-block cluster of L CTAs per tree node,
-//     CTA l on limb l, the CRT of the Dcp reading the other limb's residues
-//     through distributed shared memory (see ntt.cuh and coltor.cu); about
-//     81 KB of shared memory per CTA at N = 4096;
-//   - expand_split_kernel: for stages with few nodes, L ell CTAs per node
+//     CTA l on limb l; the CRT of the Dcp takes the other limb's residues,
+//     pushed through distributed shared memory. The limb's two polynomials are
+//     brought into shared memory whole: tau(a) and tau(b) are gathers of odd
+//     slot stride, which shared memory serves without bank conflicts (from
+//     global memory each gather of a warp touched 32 lines), and the same copy
+//     serves c's own slots at the end. All digit polynomials go through the
+//     forward transform together (see ntt.cuh), and the multiply-accumulate
+//     starts when they are done, so its 64-bit sums live for one slot at a
+//     time: 64 registers, 82 KB of shared memory at N = 4096, two CTAs per SM;
+//     Bound by instruction issue (2490 warp instructions a warp and node, 3440
+//     when each digit had its own transform and reduced after every round):
+//     32 clients, 274 outputs: 2.90 -> 1.99 ms;
+//   - expand_split_kernel: for stages with few nodes, L digits CTAs per node
 //     (limb x digit), each repeating the inverse NTT and doing one digit.
 // The tree runs in place in the output array: stage j reads list[k], k < 2^j,
-// and writes list[k] and list[k + 2^j]; each CTA reads only its limb of
-// list[k], and every such read comes before the barrier that precedes the
-// writes of that limb. Only
+// and writes list[k] and list[k + 2^j]; each CTA that writes reads only its
+// limb of list[k], and has all of it in shared memory before it writes. (In
+// the split kernel the cluster barriers order every CTA's read of tau(a)
+// before the writes.) Only
 // the outputs with index < n_out are computed at any stage (an intermediate
 // list[k] feeds final outputs k, k + 2^(j+1), ..., so k < n_out is exactly the
 // condition for it to be needed).
@@ -43,6 +53,7 @@
 #include "common.cuh"
 #include "internal.h"
 #include "ntt.cuh"
+#include "tcgen05.cuh"
 
 namespace gpir {
 namespace {
@@ -54,294 +65,293 @@ struct ExpandParams {
   uint32_t *out;                                  // [B][n_out][2][L][N]
   uint32_t n_out, J, stage, nodes;                // nodes = min(2^stage, n_out) per client
   uint32_t ksub;                                  // N / 2^stage + 1
+  uint32_t bulk;                                  // inputs are 16-byte aligned: bulk copies
+  unsigned int *err;
+};
+
+// One node: its client and index, inputs and outputs.
+struct ExpandNode {
+  const uint32_t *in, *evk;
+  uint32_t *out0, *out1;
+  bool has1;
 };
 
 template <int L, int LOGN>
-__global__ void __launch_bounds__(ntt::HALF, 2) expand_stage_kernel(const __grid_constant__ ExpandParams p) {
-  using namespace ntt;
-  constexpr uint32_t N = 1u << LOGN, S = N >> 3, PN = padn(N), MASK2N = 2 * N - 1;
-  extern __shared__ __align__(16) uint32_t sm[];
-  const Ring &R = p.ring;
-  const uint32_t ell = R.ell;
-  const uint32_t h = L > 1 ? cluster_rank() : 0u;  // this CTA's limb
-  const uint32_t b = threadIdx.x;
-  const bool act = b < S;
-  const Limb &T = R.limb[h];
-  const uint32_t q = T.q;
-  uint32_t *res = sm;                                             // [PN]: coefficients of tau(a), limb h
-  int64_t *ybuf = reinterpret_cast<int64_t *>(sm + PN + (PN & 1)); // [N]: Dcp offset values
-  uint32_t *work = sm + PN + (PN & 1) + 2 * N;                    // [2][PN]: two digit buffers
-
-  const uint32_t node = blockIdx.x / L;
-  const uint32_t c = node / p.nodes, k = node % p.nodes;
-  const size_t ctw = (size_t)2 * L * N;
-  // Plain loads: at stages >= 1 this CTA overwrites (its limb of) its input at the end.
-  const uint32_t *in = p.stage == 0 ? p.query + (size_t)c * ctw : p.out + ((size_t)c * p.n_out + k) * ctw;
-  uint32_t *out0 = p.out + ((size_t)c * p.n_out + k) * ctw;
-  const uint32_t k1 = k + (1u << p.stage);
-  const bool has1 = k1 < p.n_out;
-  uint32_t *out1 = p.out + ((size_t)c * p.n_out + k1) * ctw;
-  const uint32_t *evk = p.evk + ((size_t)c * p.J + p.stage) * ell * ctw;
-
-  // 1. tau(a) on the owned slots of limb h (a gather), then its inverse NTT
-  {
-    uint32_t v[1][8];
-    if (act) {
-#pragma unroll
-      for (uint32_t e = 0; e < 8; ++e) {
-        const uint32_t s = b + e * S;
-        const uint32_t src = ((((2 * s + 1) * p.ksub) & MASK2N) - 1) >> 1;
-        v[0][e] = in[(size_t)h * N + src];
-      }
-    }
-    uint32_t *const bufs[1] = {res};
-    inverse<LOGN, 1>(v, bufs, T, b, act);
-  }
-  if constexpr (L > 1) {
-    cluster_arrive();   // the other limb's residues are complete and visible after this pair
-    cluster_wait();
-  }
-
-  // 2a. Dcp offset values of the owned coefficients (CRT over both limbs)
-  if (act) {
-    const uint32_t peer = L > 1 ? peer_addr(res, h ^ 1u) : 0u;
-#pragma unroll
-    for (uint32_t kk = 0; kk < 8; ++kk) {
-      const uint32_t j = pad(b) + kk * S + ((kk * S) >> 7);
-      const uint32_t own = res[j];
-      uint32_t r0 = own, r1 = 0u;
-      if constexpr (L > 1) {
-        const uint32_t other = ld_peer(peer + 4 * j);
-        r0 = h == 0 ? own : other;
-        r1 = h == 0 ? other : own;
-      }
-      ybuf[b + kk * S] = dcp_offset_value(R, r0, r1);   // read back by this thread only
-    }
-  }
-  if constexpr (L > 1) cluster_arrive();   // done reading the other CTA's shared memory
-
-  // 2b. per digit: digit residues, forward NTT, multiply-accumulate with the key rows
-  uint64_t acc[2][8];
-#pragma unroll
-  for (int r = 0; r < 2; ++r)
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[r][e] = 0;
-  uint32_t ping = 0;
-  for (uint32_t i = 0; i < ell; ++i) {
-    uint32_t d[1][8];
-    if (act) {
-#pragma unroll
-      for (uint32_t kk = 0; kk < 8; ++kk) d[0][kk] = dcp_digit(ybuf[b + kk * S], i, ell, q);
-    }
-    if (act && (b & 31) < 16) {   // the 16 key-row lines this warp multiplies with after the transform
-      const uint32_t l = b & 31;
-      prefetch_l1(evk + (size_t)i * ctw + (size_t)h * N + (b & ~31u) + (l >> 3) * (size_t)L * N + (l & 7) * S);
-    }
-    {
-      uint32_t *const bufs[1] = {work + ping * PN};
-      forward<LOGN, 1>(d, bufs, T, b, act);
-    }
-    ping ^= 1;
-    if (act) {
-      const uint32_t *row = evk + (size_t)i * ctw + (size_t)h * N + b;
-#pragma unroll
-      for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int e = 0; e < 8; ++e) acc[r][e] += (uint64_t)d[0][e] * __ldg(row + (size_t)r * L * N + e * S);
-    }
-  }
-
-  // 3. t = (a', tau(b) + b'); out0 = c + t, out1 = X^(-2^j) (c - t), limb h
-  uint32_t ta[8], tb[8], ca[8], cb[8];
-  if (act) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      ta[e] = reduce64(acc[0][e], q, T.mu);
-      tb[e] = reduce64(acc[1][e], q, T.mu);
-    }
-#pragma unroll
-    for (uint32_t e = 0; e < 8; ++e) {
-      const uint32_t s = b + e * S;
-      const uint32_t src = ((((2 * s + 1) * p.ksub) & MASK2N) - 1) >> 1;
-      tb[e] = add_mod(tb[e], in[(size_t)(L + h) * N + src], q);
-      ca[e] = in[(size_t)h * N + s];
-      cb[e] = in[(size_t)(L + h) * N + s];
-    }
-  }
-  __syncthreads();   // every read of (limb h of) list[k] by this CTA precedes the writes below
-  if (act) {
-#pragma unroll
-    for (uint32_t e = 0; e < 8; ++e) {
-      const uint32_t s = b + e * S;
-      out0[(size_t)h * N + s] = add_mod(ca[e], ta[e], q);
-      out0[(size_t)(L + h) * N + s] = add_mod(cb[e], tb[e], q);
-      if (has1) {
-        const uint2 m = __ldg(T.mono + (((2 * s + 1) << p.stage) & MASK2N));
-        out1[(size_t)h * N + s] = shoup(sub_mod(ca[e], ta[e], q), m.x, m.y, q);
-        out1[(size_t)(L + h) * N + s] = shoup(sub_mod(cb[e], tb[e], q), m.x, m.y, q);
-      }
-    }
-  }
-  if constexpr (L > 1) cluster_wait();   // the other CTA has finished reading this CTA's residues
+__device__ __forceinline__ ExpandNode expand_node(const ExpandParams &p, uint32_t node) {
+  constexpr uint32_t ctw = 2 * L << LOGN;
+  const uint32_t c = node / p.nodes, k = node % p.nodes, k1 = k + (1u << p.stage);
+  uint32_t *list = p.out + (size_t)c * p.n_out * ctw;
+  ExpandNode n;
+  n.in = p.stage == 0 ? p.query + (size_t)c * ctw : list + (size_t)k * ctw;
+  n.out0 = list + (size_t)k * ctw;
+  n.out1 = list + (size_t)k1 * ctw;
+  n.has1 = k1 < p.n_out;
+  n.evk = p.evk + ((size_t)c * p.J + p.stage) * p.ring.ell * ctw;
+  return n;
 }
 
+// Limb h of the node's polynomials a and b into shared memory (a at `stage`,
+// b at `stage` + N), visible to the whole CTA on return.
+template <int L, int LOGN>
+__device__ __forceinline__ void expand_load(const ExpandParams &p, const ExpandNode &n, uint32_t h, uint32_t *stage,
+                                            uint64_t *bar) {
+  constexpr uint32_t N = 1u << LOGN;
+  if (p.bulk) {
+    if (threadIdx.x == 0) {
+      mbar_init(bar, 1);
+      fence_mbar_init();
+      mbar_arrive_expect_tx(bar, 8 * N);
+      bulk_g2s(stage, n.in + (size_t)h * N, 4 * N, bar);
+      bulk_g2s(stage + N, n.in + (size_t)(L + h) * N, 4 * N, bar);
+    }
+    __syncthreads();
+    // on expiry the copies may still be in flight: one more bounded wait
+    if (!mbar_wait_bounded(bar, 0, p.err, kErrTmaWait)) mbar_wait_bounded(bar, 0, nullptr, 0);
+  } else {
+    for (uint32_t s = threadIdx.x; s < N; s += blockDim.x) {
+      stage[s] = n.in[(size_t)h * N + s];
+      stage[N + s] = n.in[(size_t)(L + h) * N + s];
+    }
+    __syncthreads();
+  }
+}
+
+// Slot of A that holds slot b of tau(A) (2 src + 1 = (2b + 1) ksub mod 2N), and
+// the step of src from slot b + (N/8) e to the next e.
 template <int LOGN>
+__device__ __forceinline__ void tau_slots(uint32_t ksub, uint32_t b, uint32_t &src, uint32_t &step) {
+  constexpr uint32_t N = 1u << LOGN;
+  src = (b * ksub + (ksub >> 1)) & (N - 1);
+  step = ((N >> 3) * ksub) & (N - 1);
+}
+
+// The node's outputs on limb h from t = (a', b') without tau(b): out0 = c + t
+// and out1 = X^(-2^j) (c - t) on the owned slots. sum(r, e) returns
+// (64-bit) component r of t at slot b + (N/8) e. With s = c + t in [0, 4q),
+// c - t is 2c - s.
+template <int L, int LOGN, class Sum>
+__device__ __forceinline__ void expand_outputs(const ExpandParams &p, const ExpandNode &n, uint32_t h, uint32_t b,
+                                               const uint32_t *stage, const Sum &sum) {
+  using namespace ntt;
+  constexpr uint32_t N = 1u << LOGN, S = N >> 3, MASK2N = 2 * N - 1;
+  const Limb &T = p.ring.limb[h];
+  const uint32_t q = T.q;
+  uint32_t src, step;
+  tau_slots<LOGN>(p.ksub, b, src, step);
+  const uint32_t e0 = ((2 * b + 1) << p.stage) & MASK2N;
+  uint2 m = __ldg(T.mono + e0);
+  const bool early = p.stage < 3;
+#pragma unroll
+  for (uint32_t e = 0; e < 8; ++e) {
+    const uint32_t s = b + e * S;
+    // the exponent (2s + 1) 2^j mod 2N does not depend on e from stage 3 on
+    if (e > 0 && early) m = __ldg(T.mono + ((e0 + (2 * S * e << p.stage)) & MASK2N));
+    const uint32_t tb = stage[N + src];
+    src = (src + step) & (N - 1);
+#pragma unroll
+    for (uint32_t r = 0; r < 2; ++r) {
+      const uint32_t c = stage[r * N + s];
+      const uint32_t x = red64(sum(r, e) + (r == 0 ? c : c + tb), T);
+      n.out0[(size_t)(r * L + h) * N + s] = csub4(x, q);
+      if (n.has1) n.out1[(size_t)(r * L + h) * N + s] = shoup(2 * c + 4 * q - x, m, q);
+    }
+  }
+}
+
+template <int L, int LOGN>
+__global__ void __launch_bounds__(ntt::threads<LOGN>(), ntt::ctas_per_sm<LOGN>())
+    expand_stage_kernel(const __grid_constant__ ExpandParams p) {
+  using namespace ntt;
+  constexpr uint32_t N = 1u << LOGN, S = N >> 3, PN = padn(N);
+  constexpr int D = digits<L>();
+  extern __shared__ __align__(16) uint32_t sm[];
+  __shared__ uint64_t bar;
+  const uint32_t h = L > 1 ? ntt::cluster_rank() : 0u;  // this CTA's limb
+  const uint32_t b = threadIdx.x;
+  const bool act = b < S;
+  const Limb &T = p.ring.limb[h];
+  uint32_t *stage = sm;                            // [2][N]: a, b on limb h
+  uint32_t *work = sm + 2 * N;                     // [D][PN]: transforms; the last one also receives residues
+  const ExpandNode node = expand_node<L, LOGN>(p, blockIdx.x / L);
+  if constexpr (L > 1) cluster_arrive();           // this CTA runs: its peer may push into it after the wait
+  expand_load<L, LOGN>(p, node, h, stage, &bar);
+
+  // 1. tau(a) on the owned slots, then its inverse NTT
+  uint32_t a[1][8];
+  if (act) {
+    uint32_t src, step;
+    tau_slots<LOGN>(p.ksub, b, src, step);
+#pragma unroll
+    for (uint32_t e = 0; e < 8; ++e) {
+      a[0][e] = stage[src];
+      src = (src + step) & (N - 1);
+    }
+  }
+  inverse<LOGN>(a, work, T, b, act);
+
+  // 2. the other limb's residues of the owned coefficients, and the digits.
+  // They arrive where this thread's first forward round will write, so no
+  // other thread can overwrite them before they are read.
+  uint32_t *inbox = work + (D - 1) * PN + pad(b);
+  if constexpr (L > 1) {
+    cluster_wait();
+    if (act) {
+      const uint32_t to = peer_addr(inbox, h ^ 1u);
+#pragma unroll
+      for (uint32_t k = 0; k < 8; ++k) st_peer(to + 4 * pad(k * S), a[0][k]);
+    }
+    cluster_arrive();
+    cluster_wait();
+  }
+  uint32_t d[D][8];
+  if (act) {
+#pragma unroll
+    for (uint32_t k = 0; k < 8; ++k) {
+      const uint32_t own = a[0][k], other = L > 1 ? inbox[pad(k * S)] : 0u;
+      uint32_t x[D];
+      dcp_digits<L>(p.ring, T, h == 0 ? own : other, h == 0 ? other : own, x);
+#pragma unroll
+      for (int i = 0; i < D; ++i) d[i][k] = x[i];
+    }
+  }
+
+  // 3. forward NTT of the digits, multiply-accumulate with the key rows, outputs
+  {
+    uint32_t *bufs[D];
+#pragma unroll
+    for (int i = 0; i < D; ++i) bufs[i] = work + i * PN;
+    forward<LOGN, D>(d, bufs, T, b, act);
+  }
+  if (!act) return;
+  const uint32_t *row = node.evk + (size_t)h * N + b;
+  const uint32_t ell = p.ring.ell;
+  expand_outputs<L, LOGN>(p, node, h, b, stage, [&](uint32_t r, uint32_t e) {
+    uint64_t acc = 0;
+#pragma unroll
+    for (uint32_t i = 0; i < D; ++i)   // absent digits are zero: row 0 stands in for theirs
+      acc += (uint64_t)d[i][e] * __ldg(row + (size_t)(((i < ell ? i : 0u) * 2 + r) * L) * N + e * S);
+    return acc;
+  });
+}
+
+template <int L, int LOGN>
 constexpr size_t expand_smem() {
   constexpr uint32_t N = 1u << LOGN, PN = ntt::padn(N);
-  return (size_t)(PN + (PN & 1) + 2 * N + 2 * PN) * 4;
+  return (size_t)(2 * N + ntt::digits<L>() * PN) * 4;
 }
 
 // The same node for the stages with few nodes (the early ones): one cluster of
-// L ell CTAs, CTA (l, g) on limb l and digit g. Every CTA takes the inverse
-// NTT of tau(a) (repeated across g: free while the GPU is not full), then one
-// digit's forward NTT and multiply-accumulate; the digit-0 CTA of each limb
-// adds the other digits' reduced partial sums (read through distributed shared
-// memory) and writes the node's outputs.
+// L D CTAs (D = digits<L>()), CTA (l, g) on limb l and digit g. Every CTA takes
+// the inverse NTT of tau(a) (repeated across g: free while the GPU is not
+// full), then one digit's forward NTT and multiply-accumulate; the digit-0 CTA
+// of each limb receives the other digits' partial sums and writes the node's
+// outputs.
 template <int L, int LOGN>
-__global__ void __launch_bounds__(ntt::HALF, 2) expand_split_kernel(const __grid_constant__ ExpandParams p) {
+__global__ void __launch_bounds__(ntt::threads<LOGN>(), 1)
+    expand_split_kernel(const __grid_constant__ ExpandParams p) {
   using namespace ntt;
-  constexpr uint32_t N = 1u << LOGN, S = N >> 3, PN = padn(N), MASK2N = 2 * N - 1;
+  constexpr uint32_t N = 1u << LOGN, S = N >> 3, PN = padn(N);
+  constexpr int D = digits<L>();
   extern __shared__ __align__(16) uint32_t sm[];
-  const Ring &R = p.ring;
-  const uint32_t ell = R.ell;
-  const uint32_t rank = cluster_rank();
+  __shared__ uint64_t bar;
+  const uint32_t rank = ntt::cluster_rank();
   const uint32_t h = rank % L, g = rank / L;       // this CTA's limb and digit
   const uint32_t b = threadIdx.x;
   const bool act = b < S;
-  const Limb &T = R.limb[h];
-  const uint32_t q = T.q;
-  uint32_t *res = sm;                                             // [PN]: coefficients of tau(a), limb h
-  int64_t *ybuf = reinterpret_cast<int64_t *>(sm + PN + (PN & 1)); // [N]: Dcp offset values, then partial sums
-  uint32_t *work = sm + PN + (PN & 1) + 2 * N;                    // [PN]: the digit transform
-
-  const uint32_t node = blockIdx.x / (L * ell);
-  const uint32_t c = node / p.nodes, k = node % p.nodes;
-  const size_t ctw = (size_t)2 * L * N;
-  // Plain loads: at stages >= 1 the digit-0 CTAs overwrite the input at the end.
-  const uint32_t *in = p.stage == 0 ? p.query + (size_t)c * ctw : p.out + ((size_t)c * p.n_out + k) * ctw;
-  uint32_t *out0 = p.out + ((size_t)c * p.n_out + k) * ctw;
-  const uint32_t k1 = k + (1u << p.stage);
-  const bool has1 = k1 < p.n_out;
-  uint32_t *out1 = p.out + ((size_t)c * p.n_out + k1) * ctw;
-  const uint32_t *row = p.evk + ((size_t)c * p.J + p.stage) * ell * ctw + (size_t)g * ctw + (size_t)h * N;
+  const Limb &T = p.ring.limb[h];
+  const uint32_t ell = p.ring.ell;
+  uint32_t *stage = sm;                            // [2][N]: a, b on limb h
+  uint32_t *work = sm + 2 * N;                     // [PN]: transforms
+  uint32_t *inbox = work + PN + pad(b);            // [PN]: the other limb's residues
+  uint32_t *sums = work + 2 * PN;                  // [D - 1][2 N]: the other digits' partial sums (digit-0 CTAs)
+  const ExpandNode node = expand_node<L, LOGN>(p, blockIdx.x / (L * D));
+  cluster_arrive();
+  // the key values this thread multiplies with, early: they come from DRAM
+  uint32_t key[2][8];
+  if (act) {
+    const uint32_t *row = node.evk + (size_t)((g < ell ? g : 0u) * 2 * L + h) * N + b;
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) key[r][e] = __ldg(row + (size_t)r * L * N + e * S);
+  }
+  expand_load<L, LOGN>(p, node, h, stage, &bar);
 
   // 1. tau(a) on the owned slots of limb h, then its inverse NTT
-  {
-    uint32_t v[1][8];
-    if (act) {
+  uint32_t a[1][8];
+  if (act) {
+    uint32_t src, step;
+    tau_slots<LOGN>(p.ksub, b, src, step);
 #pragma unroll
-      for (uint32_t e = 0; e < 8; ++e) {
-        const uint32_t s = b + e * S;
-        const uint32_t src = ((((2 * s + 1) * p.ksub) & MASK2N) - 1) >> 1;
-        v[0][e] = in[(size_t)h * N + src];
-      }
+    for (uint32_t e = 0; e < 8; ++e) {
+      a[0][e] = stage[src];
+      src = (src + step) & (N - 1);
     }
-    uint32_t *const bufs[1] = {res};
-    inverse<LOGN, 1>(v, bufs, T, b, act);
   }
-  cluster_arrive();   // every CTA's residues are complete and visible after this pair
-  cluster_wait();
+  inverse<LOGN>(a, work, T, b, act);
+  cluster_wait();   // every CTA of the cluster runs
+  if constexpr (L > 1) {
+    if (act) {
+      const uint32_t to = peer_addr(inbox, (h ^ 1u) + L * g);
+#pragma unroll
+      for (uint32_t k = 0; k < 8; ++k) st_peer(to + 4 * pad(k * S), a[0][k]);
+    }
+    cluster_arrive();
+    cluster_wait();
+  }
 
-  // 2. digit g of the owned coefficients (CRT over the limbs), forward NTT,
-  // multiply-accumulate with key row g
+  // 2. digit g of the owned coefficients, forward NTT, product with key row g
   uint32_t d[1][8];
   if (act) {
-    const uint32_t peer = L > 1 ? peer_addr(res, (h ^ 1u) + L * g) : 0u;
 #pragma unroll
-    for (uint32_t kk = 0; kk < 8; ++kk) {
-      const uint32_t j = pad(b) + kk * S + ((kk * S) >> 7);
-      const uint32_t own = res[j];
-      uint32_t r0 = own, r1 = 0u;
-      if constexpr (L > 1) {
-        const uint32_t other = ld_peer(peer + 4 * j);
-        r0 = h == 0 ? own : other;
-        r1 = h == 0 ? other : own;
-      }
-      d[0][kk] = dcp_digit(dcp_offset_value(R, r0, r1), g, ell, q);
-    }
-    if ((b & 31) < 16) {
-      const uint32_t l = b & 31;
-      prefetch_l1(row + (b & ~31u) + (l >> 3) * (size_t)L * N + (l & 7) * S);
+    for (uint32_t k = 0; k < 8; ++k) {
+      const uint32_t own = a[0][k], other = L > 1 ? inbox[pad(k * S)] : 0u;
+      uint32_t x[D];
+      dcp_digits<L>(p.ring, T, h == 0 ? own : other, h == 0 ? other : own, x);
+      d[0][k] = x[0];
+#pragma unroll
+      for (uint32_t i = 1; i < D; ++i) d[0][k] = g == i ? x[i] : d[0][k];
     }
   }
-  cluster_arrive();   // done reading the other limb's residues
   {
     uint32_t *const bufs[1] = {work};
     forward<LOGN, 1>(d, bufs, T, b, act);
   }
-  uint32_t part[2][8];
-  if (act) {
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-      for (int e = 0; e < 8; ++e)
-        part[r][e] = reduce64((uint64_t)d[0][e] * __ldg(row + (size_t)r * L * N + b + e * S), q, T.mu);
-  }
-  uint32_t *pbuf = reinterpret_cast<uint32_t *>(ybuf);   // 2N words, unused by this kernel until now
   if (g > 0 && act) {
+    const uint32_t to = peer_addr(sums + (g - 1) * 2 * N + b, h);
 #pragma unroll
     for (int r = 0; r < 2; ++r)
 #pragma unroll
-      for (int e = 0; e < 8; ++e) pbuf[(r * 8 + e) * S + b] = part[r][e];
+      for (int e = 0; e < 8; ++e) st_peer(to + 4 * (r * N + e * S), red64((uint64_t)d[0][e] * key[r][e], T));
   }
-  cluster_wait();     // pairs the arrive after step 2
-  cluster_arrive();   // the partial sums are written
+  cluster_arrive();   // the partial sums have arrived after this pair
   cluster_wait();
 
-  // 3. digit-0 CTAs: t = (a', tau(b) + b'); out0 = c + t, out1 = X^(-2^j) (c - t), limb h
-  if (g == 0) {
-    uint32_t tb[8], ca[8], cb[8];
-    if (act) {
-      for (uint32_t gg = 1; gg < ell; ++gg) {
-        const uint32_t peer = peer_addr(pbuf, h + L * gg);
+  // 3. digit-0 CTAs: the node's outputs on limb h
+  if (g > 0 || !act) return;
+  expand_outputs<L, LOGN>(p, node, h, b, stage, [&](uint32_t r, uint32_t e) {
+    uint64_t acc = (uint64_t)d[0][e] * key[r][e];
 #pragma unroll
-        for (int r = 0; r < 2; ++r)
-#pragma unroll
-          for (int e = 0; e < 8; ++e) part[r][e] = add_mod(part[r][e], ld_peer(peer + 4 * ((r * 8 + e) * S + b)), q);
-      }
-#pragma unroll
-      for (uint32_t e = 0; e < 8; ++e) {
-        const uint32_t s = b + e * S;
-        const uint32_t src = ((((2 * s + 1) * p.ksub) & MASK2N) - 1) >> 1;
-        tb[e] = add_mod(part[1][e], in[(size_t)(L + h) * N + src], q);
-        ca[e] = in[(size_t)h * N + s];
-        cb[e] = in[(size_t)(L + h) * N + s];
-      }
-    }
-    __syncthreads();   // every read of (limb h of) list[k] by this CTA precedes the writes below
-    if (act) {
-#pragma unroll
-      for (uint32_t e = 0; e < 8; ++e) {
-        const uint32_t s = b + e * S;
-        out0[(size_t)h * N + s] = add_mod(ca[e], part[0][e], q);
-        out0[(size_t)(L + h) * N + s] = add_mod(cb[e], tb[e], q);
-        if (has1) {
-          const uint2 m = __ldg(T.mono + (((2 * s + 1) << p.stage) & MASK2N));
-          out1[(size_t)h * N + s] = shoup(sub_mod(ca[e], part[0][e], q), m.x, m.y, q);
-          out1[(size_t)(L + h) * N + s] = shoup(sub_mod(cb[e], tb[e], q), m.x, m.y, q);
-        }
-      }
-    }
-  }
-  cluster_arrive();   // the digit-0 CTAs have read the partial sums
-  cluster_wait();
+    for (uint32_t i = 1; i < D; ++i) acc += sums[(i - 1) * 2 * N + r * N + e * S + b];
+    return acc;
+  });
 }
 
-template <int LOGN>
+template <int L, int LOGN>
 constexpr size_t expand_split_smem() {
   constexpr uint32_t N = 1u << LOGN, PN = ntt::padn(N);
-  return (size_t)(PN + (PN & 1) + 2 * N + PN) * 4;
+  return (size_t)(2 * N + 2 * PN + (ntt::digits<L>() - 1) * 2 * N) * 4;
 }
 
 bool g_ex_attr_done[64][2][ntt::MAX_LIMBS][ntt::MAX_LOGN + 1] = {};
 std::mutex g_ex_mu;
 
-// One stage. split: one cluster of L ell CTAs per node (limb x digit), else one
+// One stage. split: one cluster of L digits<L>() CTAs per node (limb x digit), else one
 // cluster of L CTAs per node (limb).
 template <int L, int LOGN>
 int launch_stage(const ExpandParams &p, unsigned nodes, bool split, int dev, cudaStream_t s) {
   if (dev < 0 || dev >= 64) return GPIR_EINVAL;
-  const size_t smem = split ? expand_split_smem<LOGN>() : expand_smem<LOGN>();
+  const size_t smem = split ? expand_split_smem<L, LOGN>() : expand_smem<L, LOGN>();
   void (*kern)(ExpandParams) = split ? expand_split_kernel<L, LOGN> : expand_stage_kernel<L, LOGN>;
   {
     std::lock_guard<std::mutex> lk(g_ex_mu);
@@ -351,11 +361,11 @@ int launch_stage(const ExpandParams &p, unsigned nodes, bool split, int dev, cud
       g_ex_attr_done[dev][split][L - 1][LOGN] = true;
     }
   }
-  const unsigned cl = split ? L * p.ring.ell : L;
+  const unsigned cl = split ? L * ntt::digits<L>() : L;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3(nodes * cl);
-  cfg.blockDim = dim3(ntt::HALF);
+  cfg.blockDim = dim3(ntt::threads<LOGN>());
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -429,16 +439,19 @@ extern "C" int gpir_expand_query(const gpir_params_t *params, uint32_t batch, ui
   p.out = out_dev;
   p.n_out = n_out;
   p.J = stages;
+  p.bulk = (((uintptr_t)query_dev | (uintptr_t)out_dev) & 15u) == 0;
+  p.err = device_error_word();
   for (uint32_t st = 0; st < stages; ++st) {
     p.stage = st;
     p.nodes = (1u << st) < n_out ? (1u << st) : n_out;
     p.ksub = (N >> st) + 1;
     const unsigned nodes = batch * p.nodes;
     // stage-aware choice (Sec. 4.4): the limb x digit split (which repeats the
-    // inverse NTT per digit) when its L ell CTAs per node fit one CTA per SM,
-    // the limb split otherwise. Measured at N = 4096, L = 2: the split is about
-    // 10% faster per stage up to 16 nodes and slower from 32 nodes up.
-    const bool split = (uint64_t)nodes * L * ring.ell <= (uint64_t)sm_count() && ring.ell <= 4;
+    // inverse NTT per digit) when its CTAs fit one per SM, the limb split
+    // otherwise. Measured at N = 4096, L = 2: the split is about 10% faster
+    // per stage up to 16 nodes and slower from 32 nodes up.
+    const unsigned split_ctas = L * (L == 1 ? ntt::digits<1>() : ntt::digits<2>());
+    const bool split = (uint64_t)nodes * split_ctas <= (uint64_t)sm_count();
     const int tr = trace_begin(split ? "expand_stage_split" : "expand_stage", s);
     rc = L == 1 ? launch_stage_n<1>(p, nodes, split, dev, s) : launch_stage_n<2>(p, nodes, split, dev, s);
     trace_end(tr, s);

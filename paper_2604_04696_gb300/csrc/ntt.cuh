@@ -14,15 +14,24 @@
 // Arithmetic: Harvey's lazy butterflies ("Faster arithmetic for
 // number-theoretic transforms", J. Symb. Comp. 2014) with Shoup products:
 // a * w mod q for a fixed w is a*w - floor(a * w' / 2^32) * q with
-// w' = floor(w 2^32 / q), a value in [0, 2q) for any 32-bit a. Inverse values
-// stay in [0, 2q) (one conditional subtraction per butterfly). Forward values
-// are reduced below 8q once per radix round and grow by at most 2q per level,
-// so they stay below 14q; q < 2^28 keeps 14q < 2^32. A conditional
-// subtraction x >= c ? x - c : x is min(x, x - c) on unsigned values.
+// w' = floor(w 2^32 / q), a value in [0, 2q) for any 32-bit a. The transforms
+// let values grow as far as 32 bits allow (q < 2^28, so 16q <= 2^32), with
+// every bound tracked at compile time:
+//   - forward: a level adds 2q; the upper operand of a butterfly is brought
+//     below 8q only where the sum could pass 16q. From inputs below 2q that
+//     is at levels 7 and 11 of 12: one conditional subtraction per point of a
+//     4096-point transform. Outputs are below 16q;
+//   - inverse: sums double, products are below 2q; within a radix-8 round the
+//     bounds of the 8 values are 16, 8, 4, 4, 2, 2, 2, 2 (times q), and the
+//     four larger ones are brought below 2q at its end.
+// A conditional subtraction x >= c ? x - c : x is min(x, x - c) on unsigned
+// values.
 //
-// GPU mapping. A polynomial of one limb belongs to a CTA of HALF threads
-// (the kernels run one CTA per limb of a tree node, the limbs of a node in one
-// thread-block cluster). Thread b of the group owns the 8 points
+// GPU mapping. A polynomial of one limb belongs to a CTA of N/8 threads (the
+// kernels run one CTA per limb of a tree node, the limbs of a node in one
+// thread-block cluster). The digit polynomials of a node go through the
+// forward transform together, so a round's twiddles are loaded once for all of
+// them and they share its barrier. Thread b of the CTA owns the 8 points
 // b + (N/8) e, e = 0..7, in registers on both ends of a transform, so the
 // transforms chain with the coefficient-wise Dcp and the slot-wise
 // multiply-accumulate without a trip through memory:
@@ -36,14 +45,16 @@
 // of butterflies in registers, one store, one barrier. N is a template
 // parameter, so every round's geometry is a compile-time constant.
 //
-// Shared-memory layout: position x lives at word pad(x) = x + (x >> 7) of a
-// buffer of padn(N) = N + N/128 words. Every set of every round has the form
+// Shared-memory layout: position x lives at word pad(x) = x + 4 (x >> 9) of a
+// buffer of padn(N) words. Every set of every round has the form
 // base + k u with base = i 2^R u + o, o < u, and for those
-// pad(base + k u) = pad(base) + k u + (k u >> 7): one address per set, the
-// rest are immediate offsets. With the thread-to-set map of the 64i + o + 8k
-// round below, every access of every round at N = 4096 is free of bank
-// conflicts (the pad word per 128 spreads the bit-reversed sets 8 brv(b) + k
-// over all banks).
+// pad(base + k u) = pad(base) + k u + 4 (k u >> 9): one address per set, the
+// rest are immediate offsets. Four pad words per 512 keep groups of 4
+// positions 16-byte aligned, so the bit-reversed rounds (8 consecutive
+// positions per thread) move two 16-byte words, and with the thread-to-set map
+// of the 64i + o + 8k round below every access of every round at N = 4096 is
+// free of bank conflicts (8 consecutive threads of a bit-reversed round sit
+// 512 positions apart, which the pad spreads over all banks).
 #pragma once
 
 #include <stdint.h>
@@ -54,12 +65,23 @@
 namespace gpir {
 namespace ntt {
 
-constexpr int HALF = 512;                 // threads per limb polynomial (N/8 at N = 4096)
 constexpr uint32_t MAX_N = 4096;
 constexpr uint32_t MIN_N = 16;
 constexpr int MIN_LOGN = 4, MAX_LOGN = 12;
 constexpr uint32_t MAX_LIMBS = 2;
 constexpr int LOG_BASE = 22;              // gadget base z = 2^22 (the paper's)
+
+// Threads of a CTA that owns one limb polynomial (N/8 of them do transform
+// work, at least a warp), and the CTAs per SM that its 64 registers a thread
+// allow.
+template <int LOGN>
+__host__ __device__ constexpr int threads() { return LOGN >= 8 ? 1 << (LOGN - 3) : 32; }
+template <int LOGN>
+__host__ __device__ constexpr int ctas_per_sm() { return 1024 / threads<LOGN>() > 16 ? 16 : 1024 / threads<LOGN>(); }
+// Digit polynomials a node transforms together: the most that L 28-bit limbs
+// need. Smaller moduli need fewer digits; the absent ones are zero.
+template <int L>
+__host__ __device__ constexpr int digits() { return L == 1 ? 2 : 3; }
 
 struct Limb {
   const uint2 *fw;        // [N]  (psi^brv(k), Shoup quotient)
@@ -67,107 +89,151 @@ struct Limb {
   const uint2 *fw_last;   // [N/8][8]: the twiddles of the last forward round of thread b, in thread order
   const uint2 *iv_first;  // [N/8][8]: the twiddles of the first inverse round of thread b, in thread order
   const uint2 *mono;      // [2N] (psi^-e, Shoup quotient): slot s of NTT(X^-m) is psi^-((2s+1) m mod 2N)
-  uint32_t q, n_inv, n_inv_s, pad;
-  uint64_t mu;            // floor(2^64 / q)
+  uint2 fw8[8];           // fw[1..7] at 1..7: the first forward round, the same for every thread
+  uint2 iv8[8];           // iv[4..7], iv[2..3], iv[1] / N at 0..6: the last inverse round with its scaling
+  uint2 n_inv;            // 1 / N mod q and its Shoup quotient
+  uint2 r32;              // 2^32 mod q and its Shoup quotient
+  uint32_t q, one_s;      // one_s = floor(2^32 / q): the Shoup quotient of 1
+  uint32_t digit_add[3];  // added to the masked digit field i: minus its offset plus a multiple of q, >= 0
 };
 
 struct Ring {
   uint32_t L, N, logn, ell;
-  uint64_t Q;             // prod q_l (< 2^56)
-  uint64_t half_Q;        // floor(Q / 2)
-  uint64_t offset;        // O = sum_{k < ell-1} 2^21 2^(22 k): y = x + O has the balanced digits as plain digits
-  uint32_t q0_inv, q0_inv_s;   // q0^-1 mod q1 and its Shoup quotient (L = 2)
+  uint64_t half_Q;        // floor(Q / 2), Q = prod q_l (< 2^56)
+  uint64_t off_pos, off_neg;   // O and O - Q, O = sum_{k < ell-1} 2^21 2^(22 k): y = centred x + O
+  uint32_t digit_mask[3]; // field i of y: 22 bits below the top digit, all bits for it, 0 past it
+  uint32_t crt_add;       // multiple of q1, >= q0
+  uint2 q0_inv;           // q0^-1 mod q1 and its Shoup quotient (L = 2)
   Limb limb[MAX_LIMBS];
 };
 
-__host__ __device__ constexpr uint32_t padn(uint32_t n) { return n + (n >> 7); }
-__device__ __forceinline__ uint32_t pad(uint32_t x) { return x + (x >> 7); }
+__host__ __device__ constexpr uint32_t padn(uint32_t n) { return n + 4 * (n >> 9); }
+__host__ __device__ constexpr uint32_t pad(uint32_t x) { return x + 4 * (x >> 9); }
 __device__ __forceinline__ uint32_t brev(uint32_t x, uint32_t bits) { return bits ? __brev(x) >> (32 - bits) : 0u; }
 
 __device__ __forceinline__ uint32_t csub(uint32_t x, uint32_t c) { return min(x, x - c); }
-__device__ __forceinline__ uint32_t shoup_lazy(uint32_t a, uint32_t w, uint32_t ws, uint32_t q) {
-  return a * w - __umulhi(a, ws) * q;
+__device__ __forceinline__ uint32_t shoup_lazy(uint32_t a, uint2 w, uint32_t q) {
+  return a * w.x - __umulhi(a, w.y) * q;
 }
-__device__ __forceinline__ uint32_t shoup(uint32_t a, uint32_t w, uint32_t ws, uint32_t q) {
-  return csub(shoup_lazy(a, w, ws, q), q);
+__device__ __forceinline__ uint32_t shoup(uint32_t a, uint2 w, uint32_t q) { return csub(shoup_lazy(a, w, q), q); }
+// Any 32-bit x to [0, 2q): Shoup's product by 1.
+__device__ __forceinline__ uint32_t red32(uint32_t x, const Limb &T) { return x - __umulhi(x, T.one_s) * T.q; }
+// Any 64-bit x to [0, 4q): hi 2^32 + lo by two Shoup products, of 2^32 and of
+// 1, whose quotients are summed before the one product by q.
+__device__ __forceinline__ uint32_t red64(uint64_t x, const Limb &T) {
+  const uint32_t hi = (uint32_t)(x >> 32), lo = (uint32_t)x;
+  return hi * T.r32.x + lo - (__umulhi(hi, T.r32.y) + __umulhi(lo, T.one_s)) * T.q;
 }
-__device__ __forceinline__ uint32_t add_mod(uint32_t a, uint32_t b, uint32_t q) { return csub(a + b, q); }
-__device__ __forceinline__ uint32_t sub_mod(uint32_t a, uint32_t b, uint32_t q) { return csub(a - b + q, q); }
-
-// Cooley-Tukey butterfly with no reduction of its own: t = w y mod q lies in
-// [0, 2q) for any 32-bit y (Shoup), so x < B gives outputs below B + 2q. Each
-// forward round first brings its values below 8q (fwd_entry), so after its at
-// most three levels they stay below 14q < 2^32 (q < 2^28): one conditional
-// subtraction per value and round instead of one per butterfly.
-__device__ __forceinline__ void ct(uint32_t &x, uint32_t &y, uint32_t w, uint32_t ws, uint32_t q) {
-  const uint32_t t = shoup_lazy(y, w, ws, q);
-  const uint32_t u = x;
-  x = u + t;
-  y = u - t + 2 * q;
-}
-// Start of a forward round: values below 16q (14q from the previous round,
-// q for the input coefficients) are brought below 8q.
-template <int K>
-__device__ __forceinline__ void fwd_entry(uint32_t (&v)[8], uint32_t q) {
-#pragma unroll
-  for (int k = 0; k < K; ++k) v[k] = csub(v[k], 8 * q);
-}
-// Gentleman-Sande butterfly, inputs and outputs in [0, 2q).
-__device__ __forceinline__ void gs(uint32_t &x, uint32_t &y, uint32_t w, uint32_t ws, uint32_t q) {
-  const uint32_t u = csub(x + y, 2 * q);
-  const uint32_t t = x - y + 2 * q;
-  x = u;
-  y = shoup_lazy(t, w, ws, q);
-}
+// [0, 4q) to [0, q).
+__device__ __forceinline__ uint32_t csub4(uint32_t x, uint32_t q) { return csub(csub(x, 2 * q), q); }
 
 __device__ __forceinline__ uint4 ld4(const uint2 *p) { return __ldg(reinterpret_cast<const uint4 *>(p)); }
 __device__ __forceinline__ uint2 ld2(const uint2 *p) { return __ldg(p); }
 
-// Forward round of R levels starting at level l0 (M0 = 2^l0 groups) on the set
-// of group i: v[k] holds position i * 2^R u + o + k u, u = N / (2^R M0).
-// Level r pairs k with k + 2^(R-1-r) and uses twiddle 2^r M0 + 2^r i + (k >> (R-r)).
-template <int R, uint32_t M0>
-__device__ __forceinline__ void fwd_round(uint32_t (&v)[8], const uint2 *fw, uint32_t i, uint32_t q) {
-  fwd_entry<(1 << R)>(v, q);
-  if constexpr (R == 3) {
-    const uint2 a = ld2(fw + i + M0);
-    ct(v[0], v[4], a.x, a.y, q); ct(v[1], v[5], a.x, a.y, q); ct(v[2], v[6], a.x, a.y, q); ct(v[3], v[7], a.x, a.y, q);
-    const uint4 b = ld4(fw + 2 * i + 2 * M0);
-    ct(v[0], v[2], b.x, b.y, q); ct(v[1], v[3], b.x, b.y, q); ct(v[4], v[6], b.z, b.w, q); ct(v[5], v[7], b.z, b.w, q);
-    const uint4 c = ld4(fw + 4 * i + 4 * M0), d = ld4(fw + 4 * i + 4 * M0 + 2);
-    ct(v[0], v[1], c.x, c.y, q); ct(v[2], v[3], c.z, c.w, q); ct(v[4], v[5], d.x, d.y, q); ct(v[6], v[7], d.z, d.w, q);
-  } else if constexpr (R == 2) {
-    const uint2 a = ld2(fw + i + M0);
-    ct(v[0], v[2], a.x, a.y, q); ct(v[1], v[3], a.x, a.y, q);
-    const uint4 b = ld4(fw + 2 * i + 2 * M0);
-    ct(v[0], v[1], b.x, b.y, q); ct(v[2], v[3], b.z, b.w, q);
-  } else {
-    const uint2 a = ld2(fw + i + M0);
-    ct(v[0], v[1], a.x, a.y, q);
+// Bound (in units of q) of a forward transform's values before level l, from
+// inputs below 2q: a level adds 2 and starts at 8 again where that would pass
+// 16 (levels 7 and 11). Closed forms, so that unrolled code folds them.
+__host__ __device__ constexpr int fwd_bound(int l) { return l <= 7 ? 2 + 2 * l : l <= 11 ? 2 * l - 6 : 10; }
+// Bound of value k of an inverse round before its level r, from values below
+// 2q: products are below 2q and sums double, so it counts the levels since
+// the last one that multiplied (the highest set bit of k below bit r).
+__host__ __device__ constexpr int inv_bound(int k, int r) {
+  return r == 0 || (k >> (r - 1)) & 1 ? 2 : r == 1 || (k >> (r - 2)) & 1 ? 4 : r == 2 || (k >> (r - 3)) & 1 ? 8 : 16;
+}
+
+// R forward levels (Cooley-Tukey: x, y -> x + w y, x - w y), the first of them
+// level LVL of the transform, on P polynomials. w[2^r - 1 + j] is the twiddle
+// of the pairs k with k >> (R - r) = j at level r.
+template <int R, int LVL, int P>
+__device__ __forceinline__ void fwd_levels(uint32_t (&v)[P][8], const uint2 (&w)[7], uint32_t q) {
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int span = 1 << (R - 1 - r);
+#pragma unroll
+    for (int k = 0; k < (1 << R); ++k) {
+      if (k & span) continue;
+      const uint2 tw = w[(1 << r) - 1 + (k >> (R - r))];
+#pragma unroll
+      for (int p = 0; p < P; ++p) {
+        const uint32_t t = shoup_lazy(v[p][k + span], tw, q);
+        const uint32_t u = fwd_bound(LVL + r) + 2 > 16 ? csub(v[p][k], 8 * q) : v[p][k];
+        v[p][k] = u + t;
+        v[p][k + span] = u - t + 2 * q;
+      }
+    }
   }
 }
 
-// Inverse round of R levels starting at t0: v[k] holds position
-// i * 2^R t0 + o + k t0. Level r pairs k with k + 2^r and uses twiddle
-// H0 / 2^r + 2^(R-1-r) i + (k >> (r+1)), H0 = N / (2 t0).
+// R inverse levels (Gentleman-Sande: x, y -> x + y, w (x - y)). Level r pairs
+// k with k + 2^r; w holds level 0's 2^(R-1) twiddles, then level 1's, ...
+// LAST: the transform's last round (R = 3), whose values are scaled by 1/N and
+// reduced below q (the twiddle of its last level includes the 1/N); otherwise
+// values end below 2q.
+template <int R, bool LAST, int P>
+__device__ __forceinline__ void inv_levels(uint32_t (&v)[P][8], const uint2 (&w)[7], const Limb &T) {
+  const uint32_t q = T.q;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int span = 1 << r, first = (1 << R) - (1 << (R - r));
+#pragma unroll
+    for (int k = 0; k < (1 << R); ++k) {
+      if (k & span) continue;
+      const uint2 tw = w[first + (k >> (r + 1))];
+#pragma unroll
+      for (int p = 0; p < P; ++p) {
+        const uint32_t x = v[p][k], y = v[p][k + span];
+        v[p][k] = x + y;
+        v[p][k + span] = shoup_lazy(x - y + inv_bound(k + span, r) * q, tw, q);
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < (1 << R); ++k) {
+    const int bound = inv_bound(k, R);
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      if (LAST) v[p][k] = csub(k < (1 << (R - 1)) ? shoup_lazy(v[p][k], T.n_inv, q) : v[p][k], q);
+      else if (bound > 4) v[p][k] = red32(v[p][k], T);
+      else if (bound > 2) v[p][k] = csub(v[p][k], 2 * q);
+    }
+  }
+}
+
+// Twiddles of a forward round of R levels on the set of group i, M0 = 2^l0
+// groups at its first level l0.
+template <int R, uint32_t M0>
+__device__ __forceinline__ void fwd_twiddles(uint2 (&w)[7], const uint2 *fw, uint32_t i) {
+  w[0] = ld2(fw + i + M0);
+  if constexpr (R >= 2) {
+    const uint4 b = ld4(fw + 2 * i + 2 * M0);
+    w[1] = make_uint2(b.x, b.y);
+    w[2] = make_uint2(b.z, b.w);
+  }
+  if constexpr (R == 3) {
+    const uint4 c = ld4(fw + 4 * i + 4 * M0), d = ld4(fw + 4 * i + 4 * M0 + 2);
+    w[3] = make_uint2(c.x, c.y);
+    w[4] = make_uint2(c.z, c.w);
+    w[5] = make_uint2(d.x, d.y);
+    w[6] = make_uint2(d.z, d.w);
+  }
+}
+
+// Twiddles of an inverse round of R levels on the set of group i, H0 = N/(2 t0).
 template <int R, uint32_t H0>
-__device__ __forceinline__ void inv_round(uint32_t (&v)[8], const uint2 *iv, uint32_t i, uint32_t q) {
+__device__ __forceinline__ void inv_twiddles(uint2 (&w)[7], const uint2 *iv, uint32_t i) {
   if constexpr (R == 3) {
     const uint4 a = ld4(iv + 4 * i + H0), b = ld4(iv + 4 * i + H0 + 2);
-    gs(v[0], v[1], a.x, a.y, q); gs(v[2], v[3], a.z, a.w, q); gs(v[4], v[5], b.x, b.y, q); gs(v[6], v[7], b.z, b.w, q);
-    const uint4 c = ld4(iv + 2 * i + H0 / 2);
-    gs(v[0], v[2], c.x, c.y, q); gs(v[1], v[3], c.x, c.y, q); gs(v[4], v[6], c.z, c.w, q); gs(v[5], v[7], c.z, c.w, q);
-    const uint2 d = ld2(iv + i + H0 / 4);
-    gs(v[0], v[4], d.x, d.y, q); gs(v[1], v[5], d.x, d.y, q); gs(v[2], v[6], d.x, d.y, q); gs(v[3], v[7], d.x, d.y, q);
-  } else if constexpr (R == 2) {
-    const uint4 a = ld4(iv + 2 * i + H0);
-    gs(v[0], v[1], a.x, a.y, q); gs(v[2], v[3], a.z, a.w, q);
-    const uint2 c = ld2(iv + i + H0 / 2);
-    gs(v[0], v[2], c.x, c.y, q); gs(v[1], v[3], c.x, c.y, q);
-  } else {
-    const uint2 a = ld2(iv + i + H0);
-    gs(v[0], v[1], a.x, a.y, q);
+    w[0] = make_uint2(a.x, a.y);
+    w[1] = make_uint2(a.z, a.w);
+    w[2] = make_uint2(b.x, b.y);
+    w[3] = make_uint2(b.z, b.w);
   }
+  if constexpr (R >= 2) {
+    const uint4 c = ld4(iv + 2 * i + H0 / (R == 3 ? 2 : 1));
+    w[R == 3 ? 4 : 0] = make_uint2(c.x, c.y);
+    w[R == 3 ? 5 : 1] = make_uint2(c.z, c.w);
+  }
+  w[R == 3 ? 6 : R == 2 ? 2 : 0] = ld2(iv + i + H0 / (1 << (R - 1)));
 }
 
 // The bit-reversed rounds (the last forward round and the first inverse round,
@@ -176,20 +242,22 @@ __device__ __forceinline__ void inv_round(uint32_t (&v)[8], const uint2 *iv, uin
 // each, see ring_tables.cu), so that these loads are contiguous across a warp:
 //   fw_last[b]  = W[N/8 + i], W[N/4 + 2i], W[N/4 + 2i + 1], -, W[N/2 + 4i + 0..3]
 //   iv_first[b] = V[N/2 + 4i + 0..3], V[N/4 + 2i], V[N/4 + 2i + 1], V[N/8 + i], -
-__device__ __forceinline__ void fwd_round_last(uint32_t (&v)[8], const uint2 *t, uint32_t q) {
-  fwd_entry<8>(v, q);
-  const uint4 a = ld4(t), b = ld4(t + 2);
-  ct(v[0], v[4], a.x, a.y, q); ct(v[1], v[5], a.x, a.y, q); ct(v[2], v[6], a.x, a.y, q); ct(v[3], v[7], a.x, a.y, q);
-  ct(v[0], v[2], a.z, a.w, q); ct(v[1], v[3], a.z, a.w, q); ct(v[4], v[6], b.x, b.y, q); ct(v[5], v[7], b.x, b.y, q);
-  const uint4 c = ld4(t + 4), d = ld4(t + 6);
-  ct(v[0], v[1], c.x, c.y, q); ct(v[2], v[3], c.z, c.w, q); ct(v[4], v[5], d.x, d.y, q); ct(v[6], v[7], d.z, d.w, q);
-}
-__device__ __forceinline__ void inv_round_first(uint32_t (&v)[8], const uint2 *t, uint32_t q) {
-  const uint4 a = ld4(t), b = ld4(t + 2);
-  gs(v[0], v[1], a.x, a.y, q); gs(v[2], v[3], a.z, a.w, q); gs(v[4], v[5], b.x, b.y, q); gs(v[6], v[7], b.z, b.w, q);
-  const uint4 c = ld4(t + 4), d = ld4(t + 6);
-  gs(v[0], v[2], c.x, c.y, q); gs(v[1], v[3], c.x, c.y, q); gs(v[4], v[6], c.z, c.w, q); gs(v[5], v[7], c.z, c.w, q);
-  gs(v[0], v[4], d.x, d.y, q); gs(v[1], v[5], d.x, d.y, q); gs(v[2], v[6], d.x, d.y, q); gs(v[3], v[7], d.x, d.y, q);
+__device__ __forceinline__ void thread_twiddles(uint2 (&w)[7], const uint2 *t, bool forward) {
+  const uint4 a = ld4(t), b = ld4(t + 2), c = ld4(t + 4), d = ld4(t + 6);
+  w[0] = make_uint2(a.x, a.y);
+  w[1] = make_uint2(a.z, a.w);
+  w[2] = make_uint2(b.x, b.y);
+  if (forward) {
+    w[3] = make_uint2(c.x, c.y);
+    w[4] = make_uint2(c.z, c.w);
+    w[5] = make_uint2(d.x, d.y);
+    w[6] = make_uint2(d.z, d.w);
+  } else {
+    w[3] = make_uint2(b.z, b.w);
+    w[4] = make_uint2(c.x, c.y);
+    w[5] = make_uint2(c.z, c.w);
+    w[6] = make_uint2(d.x, d.y);
+  }
 }
 
 // Levels of the next middle round when LEFT levels remain (4 -> 2 + 2, so that
@@ -214,20 +282,26 @@ __device__ __forceinline__ void set_of(uint32_t sb, uint32_t &i, uint32_t &o) {
   }
 }
 
-template <int LOGN, int R, int LVL>
-__device__ __forceinline__ void fwd_middle(uint32_t *buf, const Limb &T, uint32_t b) {
+template <int LOGN, int R, int LVL, int P>
+__device__ __forceinline__ void fwd_middle(uint32_t *const (&buf)[P], const Limb &T, uint32_t b) {
   constexpr uint32_t N = 1u << LOGN, S = N >> 3, M0 = 1u << LVL, U = N >> (LVL + R);
 #pragma unroll
   for (uint32_t t = 0; t < (N >> R) / S; ++t) {
     uint32_t i, o;
     set_of<R, U, N>(b + t * S, i, o);
-    uint32_t *p = buf + pad((i << R) * U + o);
-    uint32_t v[8];
+    const uint32_t base = pad((i << R) * U + o);
+    uint2 w[7];
+    fwd_twiddles<R, M0>(w, T.fw, i);
+    uint32_t v[P][8];
 #pragma unroll
-    for (uint32_t k = 0; k < (1u << R); ++k) v[k] = p[k * U + ((k * U) >> 7)];
-    fwd_round<R, M0>(v, T.fw, i, T.q);
+    for (int p = 0; p < P; ++p)
 #pragma unroll
-    for (uint32_t k = 0; k < (1u << R); ++k) p[k * U + ((k * U) >> 7)] = v[k];
+      for (uint32_t k = 0; k < (1u << R); ++k) v[p][k] = buf[p][base + pad(k * U)];
+    fwd_levels<R, LVL, P>(v, w, T.q);
+#pragma unroll
+    for (int p = 0; p < P; ++p)
+#pragma unroll
+      for (uint32_t k = 0; k < (1u << R); ++k) buf[p][base + pad(k * U)] = v[p][k];
   }
 }
 
@@ -239,12 +313,14 @@ __device__ __forceinline__ void inv_middle(uint32_t *buf, const Limb &T, uint32_
     uint32_t i, o;
     set_of<R, T0, N>(b + t * S, i, o);
     uint32_t *p = buf + pad((i << R) * T0 + o);
-    uint32_t v[8];
+    uint2 w[7];
+    inv_twiddles<R, N / (2 * T0)>(w, T.iv, i);
+    uint32_t v[1][8];
 #pragma unroll
-    for (uint32_t k = 0; k < (1u << R); ++k) v[k] = p[k * T0 + ((k * T0) >> 7)];
-    inv_round<R, N / (2 * T0)>(v, T.iv, i, T.q);
+    for (uint32_t k = 0; k < (1u << R); ++k) v[0][k] = p[pad(k * T0)];
+    inv_levels<R, false, 1>(v, w, T);
 #pragma unroll
-    for (uint32_t k = 0; k < (1u << R); ++k) p[k * T0 + ((k * T0) >> 7)] = v[k];
+    for (uint32_t k = 0; k < (1u << R); ++k) p[pad(k * T0)] = v[0][k];
   }
 }
 
@@ -253,62 +329,65 @@ __device__ __forceinline__ void fwd_middles(uint32_t *const (&buf)[P], const Lim
   constexpr int END = LOGN >= 6 ? LOGN - 3 : LOGN;
   if constexpr (LVL < END) {
     constexpr int R = middle_levels<END - LVL>();
-    if (act) {
-#pragma unroll
-      for (int p = 0; p < P; ++p) fwd_middle<LOGN, R, LVL>(buf[p], T, b);
-    }
+    if (act) fwd_middle<LOGN, R, LVL, P>(buf, T, b);
     __syncthreads();
     fwd_middles<LOGN, LVL + R, P>(buf, T, b, act);
   }
 }
 
-template <int LOGN, int G, int P>
-__device__ __forceinline__ void inv_middles(uint32_t *const (&buf)[P], const Limb &T, uint32_t b, bool act) {
+template <int LOGN, int G>
+__device__ __forceinline__ void inv_middles(uint32_t *buf, const Limb &T, uint32_t b, bool act) {
   constexpr int END = LOGN >= 6 ? LOGN - 3 : LOGN;
   if constexpr (G < END) {
     constexpr int R = middle_levels<END - G>();
-    if (act) {
-#pragma unroll
-      for (int p = 0; p < P; ++p) inv_middle<LOGN, R, G>(buf[p], T, b);
-    }
+    if (act) inv_middle<LOGN, R, G>(buf, T, b);
     __syncthreads();
-    inv_middles<LOGN, G + R, P>(buf, T, b, act);
+    inv_middles<LOGN, G + R>(buf, T, b, act);
   }
 }
 
 // Forward NTT of P polynomials of one limb (one padded buffer of padn(N) words
-// each). In: v[p][k] = coefficient b + (N/8) k, values < 16q. Out: v[p][e] =
-// slot b + (N/8) e, values in [0, 14q) (lazy: congruent mod q, not reduced). Every thread of the CTA must call it
-// (it holds __syncthreads); act = b < N/8. The buffers are free again once
-// the next barrier of the CTA has passed.
+// each). In: v[p][k] = coefficient b + (N/8) k, values < 2q. Out: v[p][e] =
+// slot b + (N/8) e, values in [0, 16q) (lazy: congruent mod q, not reduced).
+// Every thread of the CTA must call it (it holds __syncthreads); act = b < N/8.
+// Before its first barrier a thread writes only the positions b + (N/8) k of
+// the buffers. They are free again once the next barrier of the CTA has passed.
 template <int LOGN, int P>
 __device__ __forceinline__ void forward(uint32_t (&v)[P][8], uint32_t *const (&buf)[P], const Limb &T, uint32_t b,
                                         bool act) {
   constexpr uint32_t N = 1u << LOGN, S = N >> 3;
   if (act) {
+    uint2 w[7];
+#pragma unroll
+    for (int k = 0; k < 7; ++k) w[k] = T.fw8[k + 1];
+    fwd_levels<3, 0, P>(v, w, T.q);
     const uint32_t base = pad(b);
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
-      fwd_round<3, 1>(v[p], T.fw, 0, T.q);
+    for (int p = 0; p < P; ++p)
 #pragma unroll
-      for (uint32_t k = 0; k < 8; ++k) buf[p][base + k * S + ((k * S) >> 7)] = v[p][k];
-    }
+      for (uint32_t k = 0; k < 8; ++k) buf[p][base + pad(k * S)] = v[p][k];
   }
   __syncthreads();
   fwd_middles<LOGN, 3, P>(buf, T, b, act);
   if (!act) return;
   if constexpr (LOGN >= 6) {
-    const uint32_t i = brev(b, LOGN - 3);
-    const uint32_t base = pad(8 * i);
+    const uint32_t base = pad(8 * brev(b, LOGN - 3));
+    uint2 w[7];
+    thread_twiddles(w, T.fw_last + 8 * b, true);
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-      uint32_t w[8];
+      const uint4 x = *reinterpret_cast<const uint4 *>(buf[p] + base);
+      const uint4 y = *reinterpret_cast<const uint4 *>(buf[p] + base + 4);
+      v[p][0] = x.x, v[p][1] = x.y, v[p][2] = x.z, v[p][3] = x.w;
+      v[p][4] = y.x, v[p][5] = y.y, v[p][6] = y.z, v[p][7] = y.w;
+    }
+    fwd_levels<3, LOGN - 3, P>(v, w, T.q);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) w[k] = buf[p][base + k];
-      fwd_round_last(w, T.fw_last + 8 * b, T.q);
+    for (int p = 0; p < P; ++p) {
       // position 8i + k holds slot (N/8) brv3(k) + b
-      v[p][0] = w[0]; v[p][1] = w[4]; v[p][2] = w[2]; v[p][3] = w[6];
-      v[p][4] = w[1]; v[p][5] = w[5]; v[p][6] = w[3]; v[p][7] = w[7];
+      const uint32_t t1 = v[p][1], t3 = v[p][3];
+      v[p][1] = v[p][4], v[p][4] = t1;
+      v[p][3] = v[p][6], v[p][6] = t3;
     }
   } else {
 #pragma unroll
@@ -318,80 +397,71 @@ __device__ __forceinline__ void forward(uint32_t (&v)[P][8], uint32_t *const (&b
   }
 }
 
-// Inverse NTT of P polynomials of one limb. In: v[p][e] = slot b + (N/8) e,
-// values < 2q. Out: the canonical coefficients in buf[p] (natural order,
-// padded layout), visible to the whole CTA on return.
-template <int LOGN, int P>
-__device__ __forceinline__ void inverse(uint32_t (&v)[P][8], uint32_t *const (&buf)[P], const Limb &T, uint32_t b,
-                                        bool act) {
+// Inverse NTT of one polynomial of one limb. In: v[e] = slot b + (N/8) e,
+// values < 2q. Out: v[k] = coefficient b + (N/8) k, below q. After its last
+// barrier a thread reads only the positions b + (N/8) k of the buffer.
+template <int LOGN>
+__device__ __forceinline__ void inverse(uint32_t (&v)[1][8], uint32_t *buf, const Limb &T, uint32_t b, bool act) {
   constexpr uint32_t N = 1u << LOGN, S = N >> 3;
+  uint2 w[7];
   if (act) {
     const uint32_t i = brev(b, LOGN - 3);
-    const uint32_t base = pad(8 * i);
-#pragma unroll
-    for (int p = 0; p < P; ++p) {
-      // position 8i + k holds slot (N/8) brv3(k) + b
-      uint32_t w[8] = {v[p][0], v[p][4], v[p][2], v[p][6], v[p][1], v[p][5], v[p][3], v[p][7]};
-      if constexpr (LOGN >= 6) inv_round_first(w, T.iv_first + 8 * b, T.q);
-      else inv_round<3, (N >> 1)>(w, T.iv, i, T.q);
-#pragma unroll
-      for (int k = 0; k < 8; ++k) buf[p][base + k] = w[k];
-    }
+    if constexpr (LOGN >= 6) thread_twiddles(w, T.iv_first + 8 * b, false);
+    else inv_twiddles<3, (N >> 1)>(w, T.iv, i);
+    // position 8i + k holds slot (N/8) brv3(k) + b
+    const uint32_t t1 = v[0][1], t3 = v[0][3];
+    v[0][1] = v[0][4], v[0][4] = t1;
+    v[0][3] = v[0][6], v[0][6] = t3;
+    inv_levels<3, false, 1>(v, w, T);
+    uint4 *p = reinterpret_cast<uint4 *>(buf + pad(8 * i));
+    p[0] = make_uint4(v[0][0], v[0][1], v[0][2], v[0][3]);
+    p[1] = make_uint4(v[0][4], v[0][5], v[0][6], v[0][7]);
   }
   __syncthreads();
-  inv_middles<LOGN, 3, P>(buf, T, b, act);
-  if (act) {
-    const uint32_t base = pad(b);
+  inv_middles<LOGN, 3>(buf, T, b, act);
+  if (!act) return;
+  const uint32_t base = pad(b);
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
-      uint32_t w[8];
+  for (uint32_t k = 0; k < 8; ++k) v[0][k] = buf[base + pad(k * S)];
+  if constexpr (LOGN >= 6) {
 #pragma unroll
-      for (uint32_t k = 0; k < 8; ++k) w[k] = buf[p][base + k * S + ((k * S) >> 7)];
-      if constexpr (LOGN >= 6) inv_round<3, 4>(w, T.iv, 0, T.q);
+    for (int k = 0; k < 7; ++k) w[k] = T.iv8[k];
+    inv_levels<3, true, 1>(v, w, T);
+  } else {
 #pragma unroll
-      for (uint32_t k = 0; k < 8; ++k)
-        buf[p][base + k * S + ((k * S) >> 7)] = shoup(w[k], T.n_inv, T.n_inv_s, T.q);
-    }
+    for (uint32_t k = 0; k < 8; ++k) v[0][k] = shoup(v[0][k], T.n_inv, T.q);
   }
-  __syncthreads();
 }
 
-// Dcp, first half: y = x + O for the centred CRT value x in (-Q/2, Q/2] of one
-// coefficient with residues (r0 mod q0, r1 mod q1) (Garner for L = 2), where
+// Dcp: y = x + O for the centred CRT value x in (-Q/2, Q/2] of one coefficient
+// with residues (r0 mod q0, r1 mod q1) (Garner for L = 2), where
 // O = sum_{k < ell-1} (z/2) z^k. The balanced base-z digits of x are then
 // plain fields of y: d_k = ((y >> 22k) mod z) - z/2 for k < ell - 1, and the
-// top digit is y >> 22 (ell - 1) (arithmetic shift).
-__device__ __forceinline__ int64_t dcp_offset_value(const Ring &R, uint32_t r0, uint32_t r1) {
-  uint64_t x;
-  if (R.L == 1) {
-    x = r0;
-  } else {
+// top digit is y >> 22 (ell - 1) (arithmetic shift; its low 32 bits hold it).
+// d[i] is digit i mod q, below 2q.
+template <int L>
+__device__ __forceinline__ void dcp_digits(const Ring &R, const Limb &T, uint32_t r0, uint32_t r1,
+                                           uint32_t (&d)[digits<L>()]) {
+  uint64_t x = r0;
+  if constexpr (L > 1) {
     const uint32_t q1 = R.limb[1].q;
-    const uint32_t k = shoup(sub_mod(r1, csub(r0, q1), q1), R.q0_inv, R.q0_inv_s, q1);   // q0 < 2 q1
-    x = (uint64_t)r0 + (uint64_t)R.limb[0].q * k;
+    const uint32_t k = shoup(r1 + R.crt_add - r0, R.q0_inv, q1);
+    x += (uint64_t)R.limb[0].q * k;
   }
-  const int64_t xc = x > R.half_Q ? (int64_t)(x - R.Q) : (int64_t)x;
-  return xc + (int64_t)R.offset;
-}
-
-// Dcp, second half: digit i of y, reduced mod q (|d| < q).
-__device__ __forceinline__ uint32_t dcp_digit(int64_t y, uint32_t i, uint32_t ell, uint32_t q) {
-  constexpr int32_t z = 1 << LOG_BASE;
-  int32_t d;
-  if (i + 1 == ell) {
-    d = (int32_t)(y >> (LOG_BASE * i));
-  } else {
-    d = (int32_t)(((uint64_t)y >> (LOG_BASE * i)) & (uint64_t)(z - 1)) - z / 2;
-  }
-  return (uint32_t)d + (d < 0 ? q : 0u);
+  const uint64_t y = x + (x > R.half_Q ? R.off_neg : R.off_pos);
+#pragma unroll
+  for (int i = 0; i < digits<L>(); ++i)
+    d[i] = ((uint32_t)((int64_t)y >> (LOG_BASE * i)) & R.digit_mask[i]) + T.digit_add[i];
 }
 
 __device__ __forceinline__ void prefetch_l1(const void *p) {
   asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
 }
 
-// Thread-block cluster helpers: the two limb CTAs of a tree node exchange
-// coefficient residues through distributed shared memory.
+// Thread-block cluster helpers: the CTAs of a tree node hand each other
+// coefficient residues and partial sums through distributed shared memory.
+// They are pushed: the receiver reads its own shared memory after the barrier,
+// and no CTA has to outlive its peers' reads.
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -403,10 +473,8 @@ __device__ __forceinline__ uint32_t peer_addr(const void *local, uint32_t rank) 
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(local)), "r"(rank));
   return r;
 }
-__device__ __forceinline__ uint32_t ld_peer(uint32_t addr) {
-  uint32_t v;
-  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-  return v;
+__device__ __forceinline__ void st_peer(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 __device__ __forceinline__ void cluster_arrive() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");

@@ -96,10 +96,10 @@ static int ring_tables_impl(const gpir_params_t *params, ntt::Ring *out) {
   R.L = L;
   R.N = N;
   R.logn = logn;
-  R.Q = 1;
+  uint64_t Q = 1;
   for (uint32_t l = 0; l < L; ++l) {
     const uint64_t q = params->primes[l];
-    R.Q *= q;
+    Q *= q;
     const uint64_t psi = pow_mod(smallest_generator(q), (q - 1) / (2 * N), q);
     const uint64_t psi_inv = pow_mod(psi, q - 2, q);
     uint2 *fw = host.data() + per_limb * l, *iv = fw + N, *mono = iv + N;
@@ -131,27 +131,44 @@ static int ring_tables_impl(const gpir_params_t *params, ntt::Ring *out) {
       v[6] = iv[S + i];
       v[7] = make_uint2(0, 0);
     }
+    ntt::Limb &T = R.limb[l];
     const uint64_t ninv = pow_mod(N, q - 2, q);
-    R.limb[l].q = (uint32_t)q;
-    R.limb[l].n_inv = (uint32_t)ninv;
-    R.limb[l].n_inv_s = shoup_quotient(ninv, q);
-    R.limb[l].mu = ~0ull / q;
+    const auto shoup_pair = [q](uint64_t w) { return make_uint2((uint32_t)w, shoup_quotient(w, q)); };
+    for (uint32_t k = 1; k < 8; ++k) T.fw8[k] = fw[k];
+    for (uint32_t k = 0; k < 4; ++k) T.iv8[k] = iv[4 + k];
+    T.iv8[4] = iv[2];
+    T.iv8[5] = iv[3];
+    T.iv8[6] = shoup_pair(iv[1].x * ninv % q);
+    T.n_inv = shoup_pair(ninv);
+    T.r32 = shoup_pair((1ull << 32) % q);
+    T.q = (uint32_t)q;
+    T.one_s = shoup_quotient(1, q);
   }
   if (L == 2) {
-    const uint64_t q1 = params->primes[1];
-    const uint64_t inv = pow_mod(params->primes[0] % q1, q1 - 2, q1);
-    R.q0_inv = (uint32_t)inv;
-    R.q0_inv_s = shoup_quotient(inv, q1);
+    const uint64_t q0 = params->primes[0], q1 = params->primes[1];
+    const uint64_t inv = pow_mod(q0 % q1, q1 - 2, q1);
+    R.q0_inv = make_uint2((uint32_t)inv, shoup_quotient(inv, q1));
+    R.crt_add = (uint32_t)((q0 + q1 - 1) / q1 * q1);
   }
   {
-    unsigned __int128 Q = R.Q;
     uint32_t bits = 0;
-    for (unsigned __int128 v = Q - 1; v; v >>= 1) ++bits;
+    for (uint64_t v = Q - 1; v; v >>= 1) ++bits;
     R.ell = (bits + ntt::LOG_BASE - 1) / ntt::LOG_BASE;
   }
-  R.half_Q = R.Q / 2;
-  R.offset = 0;
-  for (uint32_t k = 0; k + 1 < R.ell; ++k) R.offset += (1ull << (ntt::LOG_BASE - 1)) << (ntt::LOG_BASE * k);
+  R.half_Q = Q / 2;
+  // digit fields below the top one carry an offset of z/2; the top digit lies
+  // in [-z/2 - 1, z/2 + 1]. Both become nonnegative by a multiple of q.
+  const uint32_t half_z = 1u << (ntt::LOG_BASE - 1);
+  for (uint32_t i = 0; i + 1 < R.ell; ++i) R.off_pos += (uint64_t)half_z << (ntt::LOG_BASE * i);
+  R.off_neg = R.off_pos - Q;
+  for (uint32_t i = 0; i < R.ell; ++i) {
+    const bool top = i + 1 == R.ell;
+    R.digit_mask[i] = top ? ~0u : 2 * half_z - 1;
+    for (uint32_t l = 0; l < L; ++l) {
+      const uint32_t q = params->primes[l], up = (half_z + 1 + q - 1) / q * q;
+      R.limb[l].digit_add[i] = top ? up : up - half_z;
+    }
+  }
   uint2 *mem = nullptr;
   e = dev_malloc(reinterpret_cast<void **>(&mem), host.size() * sizeof(uint2));
   if (e != cudaSuccess) return set_cuda_error(e);
