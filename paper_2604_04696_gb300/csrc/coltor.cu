@@ -77,15 +77,17 @@ __global__ void __launch_bounds__(ntt::threads<LOGN>(), ntt::ctas_per_sm<LOGN>()
   const uint32_t *lo = p.in + ((size_t)c * p.d_in + 2 * k) * ctw + (size_t)(pp * L + h) * N + b;
   const uint32_t *hi = lo + ctw;
   const uint32_t *row = p.rgsw + (((size_t)c * p.stages + p.stage) * 2 + pp) * ell * ctw + (size_t)h * N + b;
-  cluster_arrive();   // this CTA runs: its peers may push into it after the wait
+  cluster_arrive_relaxed();   // this CTA runs: its peers may push into it after the wait
 
   // 1. hi - lo on the owned slots of (pp, h), then its inverse NTT
   uint32_t a[1][8];
+  uint2 w[7];
   if (act) {
+    inv_first_twiddles<LOGN>(w, T, b);
 #pragma unroll
     for (int e = 0; e < 8; ++e) a[0][e] = __ldg(hi + e * S) - __ldg(lo + e * S) + q;
   }
-  inverse<LOGN>(a, work, T, b, act);
+  inverse<LOGN>(a, work, w, T, b, act);
   cluster_wait();
 
   // 2. the other limb's residues of the owned coefficients, and the digits.

@@ -63,7 +63,7 @@ struct ExpandParams {
   const uint32_t *query;                          // [B][2][L][N] (read by stage 0)
   const uint32_t *evk;                            // [B][J][ell][2][L][N]
   uint32_t *out;                                  // [B][n_out][2][L][N]
-  uint32_t n_out, J, stage, nodes;                // nodes = min(2^stage, n_out) per client
+  uint32_t batch, n_out, J, stage, nodes;         // nodes = min(2^stage, n_out) per client
   uint32_t ksub;                                  // N / 2^stage + 1
   uint32_t bulk;                                  // inputs are 16-byte aligned: bulk copies
   unsigned int *err;
@@ -129,9 +129,9 @@ __device__ __forceinline__ void tau_slots(uint32_t ksub, uint32_t b, uint32_t &s
 // and out1 = X^(-2^j) (c - t) on the owned slots. sum(r, e) returns
 // (64-bit) component r of t at slot b + (N/8) e. With s = c + t in [0, 4q),
 // c - t is 2c - s.
-template <int L, int LOGN, class Sum>
+template <int L, int LOGN, class OwnA, class Sum>
 __device__ __forceinline__ void expand_outputs(const ExpandParams &p, const ExpandNode &n, uint32_t h, uint32_t b,
-                                               const uint32_t *stage, const Sum &sum) {
+                                               const uint32_t *pb, const OwnA &own_a, const Sum &sum) {
   using namespace ntt;
   constexpr uint32_t N = 1u << LOGN, S = N >> 3, MASK2N = 2 * N - 1;
   const Limb &T = p.ring.limb[h];
@@ -146,11 +146,11 @@ __device__ __forceinline__ void expand_outputs(const ExpandParams &p, const Expa
     const uint32_t s = b + e * S;
     // the exponent (2s + 1) 2^j mod 2N does not depend on e from stage 3 on
     if (e > 0 && early) m = __ldg(T.mono + ((e0 + (2 * S * e << p.stage)) & MASK2N));
-    const uint32_t tb = stage[N + src];
+    const uint32_t tb = pb[src];
     src = (src + step) & (N - 1);
 #pragma unroll
     for (uint32_t r = 0; r < 2; ++r) {
-      const uint32_t c = stage[r * N + s];
+      const uint32_t c = r == 0 ? own_a(e) : pb[s];
       const uint32_t x = red64(sum(r, e) + (r == 0 ? c : c + tb), T);
       n.out0[(size_t)(r * L + h) * N + s] = csub4(x, q);
       if (n.has1) n.out1[(size_t)(r * L + h) * N + s] = shoup(2 * c + 4 * q - x, m, q);
@@ -158,6 +158,9 @@ __device__ __forceinline__ void expand_outputs(const ExpandParams &p, const Expa
   }
 }
 
+// Persistent: cluster i runs nodes i, i + clusters, ... Polynomial a of the next
+// node and b of the current one are copied while the current node computes, so
+// only the first node waits for its load.
 template <int L, int LOGN>
 __global__ void __launch_bounds__(ntt::threads<LOGN>(), ntt::ctas_per_sm<LOGN>())
     expand_stage_kernel(const __grid_constant__ ExpandParams p) {
@@ -165,73 +168,114 @@ __global__ void __launch_bounds__(ntt::threads<LOGN>(), ntt::ctas_per_sm<LOGN>()
   constexpr uint32_t N = 1u << LOGN, S = N >> 3, PN = padn(N);
   constexpr int D = digits<L>();
   extern __shared__ __align__(16) uint32_t sm[];
-  __shared__ uint64_t bar;
+  __shared__ uint64_t bar[2];                      // a landed, b landed
   const uint32_t h = L > 1 ? ntt::cluster_rank() : 0u;  // this CTA's limb
   const uint32_t b = threadIdx.x;
   const bool act = b < S;
   const Limb &T = p.ring.limb[h];
-  uint32_t *stage = sm;                            // [2][N]: a, b on limb h
+  uint32_t *pa = sm, *pb = sm + N;                 // [N] each: a, b on limb h
   uint32_t *work = sm + 2 * N;                     // [D][PN]: transforms; the last one also receives residues
-  const ExpandNode node = expand_node<L, LOGN>(p, blockIdx.x / L);
-  if constexpr (L > 1) cluster_arrive();           // this CTA runs: its peer may push into it after the wait
-  expand_load<L, LOGN>(p, node, h, stage, &bar);
-
-  // 1. tau(a) on the owned slots, then its inverse NTT
-  uint32_t a[1][8];
-  if (act) {
-    uint32_t src, step;
-    tau_slots<LOGN>(p.ksub, b, src, step);
-#pragma unroll
-    for (uint32_t e = 0; e < 8; ++e) {
-      a[0][e] = stage[src];
-      src = (src + step) & (N - 1);
+  const uint32_t total = p.nodes * p.batch, stride = gridDim.x / L;
+  if constexpr (L > 1) cluster_arrive_relaxed();   // this CTA runs: its peer may push into it after the wait
+  if (b == 0) {
+    mbar_init(&bar[0], 1);
+    mbar_init(&bar[1], 1);
+    fence_mbar_init();
+    if (p.bulk) {
+      mbar_arrive_expect_tx(&bar[0], 4 * N);
+      bulk_g2s(pa, expand_node<L, LOGN>(p, blockIdx.x / L).in + (size_t)h * N, 4 * N, &bar[0]);
     }
   }
-  inverse<LOGN>(a, work, T, b, act);
+  __syncthreads();
+  uint32_t ph = 0;
+  for (uint32_t i = blockIdx.x / L; i < total; i += stride, ph ^= 1) {
+    const ExpandNode node = expand_node<L, LOGN>(p, i);
+    uint2 w[7];
+    if (act) inv_first_twiddles<LOGN>(w, T, b);
+    if (p.bulk) {
+      // on expiry the copy may still be in flight: one more bounded wait
+      if (!mbar_wait_bounded(&bar[0], ph, p.err, kErrTmaWait)) mbar_wait_bounded(&bar[0], ph, nullptr, 0);
+    } else {
+      __syncthreads();   // the previous node's b has been read
+      for (uint32_t s = b; s < N; s += blockDim.x) {
+        pa[s] = node.in[(size_t)h * N + s];
+        pb[s] = node.in[(size_t)(L + h) * N + s];
+      }
+      __syncthreads();
+    }
 
-  // 2. the other limb's residues of the owned coefficients, and the digits.
-  // They arrive where this thread's first forward round will write, so no
-  // other thread can overwrite them before they are read.
-  uint32_t *inbox = work + (D - 1) * PN + pad(b);
-  if constexpr (L > 1) {
-    cluster_wait();
+    // 1. tau(a) on the owned slots, then its inverse NTT
+    uint32_t a[1][8];
     if (act) {
-      const uint32_t to = peer_addr(inbox, h ^ 1u);
+      uint32_t src, step;
+      tau_slots<LOGN>(p.ksub, b, src, step);
 #pragma unroll
-      for (uint32_t k = 0; k < 8; ++k) st_peer(to + 4 * pad(k * S), a[0][k]);
+      for (uint32_t e = 0; e < 8; ++e) {
+        a[0][e] = pa[src];
+        src = (src + step) & (N - 1);
+      }
     }
-    cluster_arrive();
-    cluster_wait();
-  }
-  uint32_t d[D][8];
-  if (act) {
-#pragma unroll
-    for (uint32_t k = 0; k < 8; ++k) {
-      const uint32_t own = a[0][k], other = L > 1 ? inbox[pad(k * S)] : 0u;
-      uint32_t x[D];
-      dcp_digits<L>(p.ring, T, h == 0 ? own : other, h == 0 ? other : own, x);
-#pragma unroll
-      for (int i = 0; i < D; ++i) d[i][k] = x[i];
+    inverse<LOGN>(a, work, w, T, b, act);
+    if (b == 0 && p.bulk) {
+      // every thread has read a, and the previous node's b, before the barriers of the transform
+      mbar_arrive_expect_tx(&bar[1], 4 * N);
+      bulk_g2s(pb, node.in + (size_t)(L + h) * N, 4 * N, &bar[1]);
+      if (i + stride < total) {
+        mbar_arrive_expect_tx(&bar[0], 4 * N);
+        bulk_g2s(pa, expand_node<L, LOGN>(p, i + stride).in + (size_t)h * N, 4 * N, &bar[0]);
+      }
     }
-  }
 
-  // 3. forward NTT of the digits, multiply-accumulate with the key rows, outputs
-  {
-    uint32_t *bufs[D];
+    // 2. the other limb's residues of the owned coefficients, and the digits.
+    // They arrive where this thread's first forward round will write, so no
+    // other thread can overwrite them before they are read.
+    uint32_t *inbox = work + (D - 1) * PN + pad(b);
+    if constexpr (L > 1) {
+      cluster_wait();
+      if (act) {
+        const uint32_t to = peer_addr(inbox, h ^ 1u);
 #pragma unroll
-    for (int i = 0; i < D; ++i) bufs[i] = work + i * PN;
-    forward<LOGN, D>(d, bufs, T, b, act);
+        for (uint32_t k = 0; k < 8; ++k) st_peer(to + 4 * pad(k * S), a[0][k]);
+      }
+      cluster_arrive();
+      cluster_wait();
+    }
+    uint32_t d[D][8];
+    if (act) {
+#pragma unroll
+      for (uint32_t k = 0; k < 8; ++k) {
+        const uint32_t own = a[0][k], other = L > 1 ? inbox[pad(k * S)] : 0u;
+        uint32_t x[D];
+        dcp_digits<L>(p.ring, T, h == 0 ? own : other, h == 0 ? other : own, x);
+#pragma unroll
+        for (int j = 0; j < D; ++j) d[j][k] = x[j];
+      }
+    }
+
+    // 3. forward NTT of the digits, multiply-accumulate with the key rows, outputs
+    const uint32_t *row = node.evk + (size_t)h * N + b;
+    const uint32_t ell = p.ring.ell;
+    {
+      uint32_t *bufs[D];
+#pragma unroll
+      for (int j = 0; j < D; ++j) bufs[j] = work + j * PN;
+      forward<LOGN, D>(d, bufs, T, b, act);
+    }
+    if (p.bulk && !mbar_wait_bounded(&bar[1], ph, p.err, kErrTmaWait)) mbar_wait_bounded(&bar[1], ph, nullptr, 0);
+    if (act) {
+      expand_outputs<L, LOGN>(
+          p, node, h, b, pb, [&](uint32_t e) { return node.in[(size_t)h * N + b + e * S]; },
+          [&](uint32_t r, uint32_t e) {
+            uint64_t acc = 0;
+#pragma unroll
+            for (uint32_t j = 0; j < D; ++j)   // absent digits are zero: row 0 stands in for theirs
+              acc += (uint64_t)d[j][e] * __ldg(row + (size_t)(((j < ell ? j : 0u) * 2 + r) * L) * N + e * S);
+            return acc;
+          });
+    }
+    if constexpr (L > 1)
+      if (i + stride < total) cluster_arrive_relaxed();   // done with this node's buffers
   }
-  if (!act) return;
-  const uint32_t *row = node.evk + (size_t)h * N + b;
-  const uint32_t ell = p.ring.ell;
-  expand_outputs<L, LOGN>(p, node, h, b, stage, [&](uint32_t r, uint32_t e) {
-    uint64_t acc = 0;
-#pragma unroll
-    for (uint32_t i = 0; i < D; ++i)   // absent digits are zero: row 0 stands in for theirs
-      acc += (uint64_t)d[i][e] * __ldg(row + (size_t)(((i < ell ? i : 0u) * 2 + r) * L) * N + e * S);
-    return acc;
-  });
 }
 
 template <int L, int LOGN>
@@ -265,7 +309,7 @@ __global__ void __launch_bounds__(ntt::threads<LOGN>(), 1)
   uint32_t *inbox = work + PN + pad(b);            // [PN]: the other limb's residues
   uint32_t *sums = work + 2 * PN;                  // [D - 1][2 N]: the other digits' partial sums (digit-0 CTAs)
   const ExpandNode node = expand_node<L, LOGN>(p, blockIdx.x / (L * D));
-  cluster_arrive();
+  cluster_arrive_relaxed();
   // the key values this thread multiplies with, early: they come from DRAM
   uint32_t key[2][8];
   if (act) {
@@ -275,6 +319,8 @@ __global__ void __launch_bounds__(ntt::threads<LOGN>(), 1)
 #pragma unroll
       for (int e = 0; e < 8; ++e) key[r][e] = __ldg(row + (size_t)r * L * N + e * S);
   }
+  uint2 w[7];
+  if (act) inv_first_twiddles<LOGN>(w, T, b);
   expand_load<L, LOGN>(p, node, h, stage, &bar);
 
   // 1. tau(a) on the owned slots of limb h, then its inverse NTT
@@ -288,7 +334,7 @@ __global__ void __launch_bounds__(ntt::threads<LOGN>(), 1)
       src = (src + step) & (N - 1);
     }
   }
-  inverse<LOGN>(a, work, T, b, act);
+  inverse<LOGN>(a, work, w, T, b, act);
   cluster_wait();   // every CTA of the cluster runs
   if constexpr (L > 1) {
     if (act) {
@@ -329,12 +375,14 @@ __global__ void __launch_bounds__(ntt::threads<LOGN>(), 1)
 
   // 3. digit-0 CTAs: the node's outputs on limb h
   if (g > 0 || !act) return;
-  expand_outputs<L, LOGN>(p, node, h, b, stage, [&](uint32_t r, uint32_t e) {
-    uint64_t acc = (uint64_t)d[0][e] * key[r][e];
+  expand_outputs<L, LOGN>(
+      p, node, h, b, stage + N, [&](uint32_t e) { return stage[b + e * S]; },
+      [&](uint32_t r, uint32_t e) {
+        uint64_t acc = (uint64_t)d[0][e] * key[r][e];
 #pragma unroll
-    for (uint32_t i = 1; i < D; ++i) acc += sums[(i - 1) * 2 * N + r * N + e * S + b];
-    return acc;
-  });
+        for (uint32_t i = 1; i < D; ++i) acc += sums[(i - 1) * 2 * N + r * N + e * S + b];
+        return acc;
+      });
 }
 
 template <int L, int LOGN>
@@ -364,7 +412,9 @@ int launch_stage(const ExpandParams &p, unsigned nodes, bool split, int dev, cud
   const unsigned cl = split ? L * ntt::digits<L>() : L;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3(nodes * cl);
+  // the limb form is persistent: as many clusters as the SMs hold
+  const unsigned resident = (unsigned)(sm_count() * ntt::ctas_per_sm<LOGN>() / L);
+  cfg.gridDim = dim3((split || nodes < resident ? nodes : resident) * cl);
   cfg.blockDim = dim3(ntt::threads<LOGN>());
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
@@ -437,6 +487,7 @@ extern "C" int gpir_expand_query(const gpir_params_t *params, uint32_t batch, ui
   p.query = query_dev;
   p.evk = evk_dev;
   p.out = out_dev;
+  p.batch = batch;
   p.n_out = n_out;
   p.J = stages;
   p.bulk = (((uintptr_t)query_dev | (uintptr_t)out_dev) & 15u) == 0;

@@ -31,7 +31,8 @@
 // kernels run one CTA per limb of a tree node, the limbs of a node in one
 // thread-block cluster). The digit polynomials of a node go through the
 // forward transform together, so a round's twiddles are loaded once for all of
-// them and they share its barrier. Thread b of the CTA owns the 8 points
+// them and they share its barrier; a round's twiddles are loaded before the
+// barrier it starts with. Thread b of the CTA owns the 8 points
 // b + (N/8) e, e = 0..7, in registers on both ends of a transform, so the
 // transforms chain with the coefficient-wise Dcp and the slot-wise
 // multiply-accumulate without a trip through memory:
@@ -94,6 +95,7 @@ struct Limb {
   uint2 n_inv;            // 1 / N mod q and its Shoup quotient
   uint2 r32;              // 2^32 mod q and its Shoup quotient
   uint32_t q, one_s;      // one_s = floor(2^32 / q): the Shoup quotient of 1
+  uint32_t q2, pad;       // 2q: kept as a value of its own, so that u - t + 2q stays one three-operand addition
   uint32_t digit_add[3];  // added to the masked digit field i: minus its offset plus a multiple of q, >= 0
 };
 
@@ -145,7 +147,8 @@ __host__ __device__ constexpr int inv_bound(int k, int r) {
 // level LVL of the transform, on P polynomials. w[2^r - 1 + j] is the twiddle
 // of the pairs k with k >> (R - r) = j at level r.
 template <int R, int LVL, int P>
-__device__ __forceinline__ void fwd_levels(uint32_t (&v)[P][8], const uint2 (&w)[7], uint32_t q) {
+__device__ __forceinline__ void fwd_levels(uint32_t (&v)[P][8], const uint2 (&w)[7], const Limb &T) {
+  const uint32_t q = T.q, q2 = T.q2;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int span = 1 << (R - 1 - r);
@@ -158,7 +161,7 @@ __device__ __forceinline__ void fwd_levels(uint32_t (&v)[P][8], const uint2 (&w)
         const uint32_t t = shoup_lazy(v[p][k + span], tw, q);
         const uint32_t u = fwd_bound(LVL + r) + 2 > 16 ? csub(v[p][k], 8 * q) : v[p][k];
         v[p][k] = u + t;
-        v[p][k + span] = u - t + 2 * q;
+        v[p][k + span] = u - t + q2;
       }
     }
   }
@@ -171,7 +174,7 @@ __device__ __forceinline__ void fwd_levels(uint32_t (&v)[P][8], const uint2 (&w)
 // values end below 2q.
 template <int R, bool LAST, int P>
 __device__ __forceinline__ void inv_levels(uint32_t (&v)[P][8], const uint2 (&w)[7], const Limb &T) {
-  const uint32_t q = T.q;
+  const uint32_t q = T.q, q2 = T.q2;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int span = 1 << r, first = (1 << R) - (1 << (R - r));
@@ -183,7 +186,7 @@ __device__ __forceinline__ void inv_levels(uint32_t (&v)[P][8], const uint2 (&w)
       for (int p = 0; p < P; ++p) {
         const uint32_t x = v[p][k], y = v[p][k + span];
         v[p][k] = x + y;
-        v[p][k + span] = shoup_lazy(x - y + inv_bound(k + span, r) * q, tw, q);
+        v[p][k + span] = shoup_lazy(x - y + (inv_bound(k + span, r) == 2 ? q2 : inv_bound(k + span, r) / 2 * q2), tw, q);
       }
     }
   }
@@ -194,7 +197,7 @@ __device__ __forceinline__ void inv_levels(uint32_t (&v)[P][8], const uint2 (&w)
     for (int p = 0; p < P; ++p) {
       if (LAST) v[p][k] = csub(k < (1 << (R - 1)) ? shoup_lazy(v[p][k], T.n_inv, q) : v[p][k], q);
       else if (bound > 4) v[p][k] = red32(v[p][k], T);
-      else if (bound > 2) v[p][k] = csub(v[p][k], 2 * q);
+      else if (bound > 2) v[p][k] = csub(v[p][k], q2);
     }
   }
 }
@@ -282,22 +285,55 @@ __device__ __forceinline__ void set_of(uint32_t sb, uint32_t &i, uint32_t &o) {
   }
 }
 
+// Levels still to do when the bit-reversed round (if the ring is large enough
+// to have one) begins.
+template <int LOGN>
+__host__ __device__ constexpr int middle_end() { return LOGN >= 6 ? LOGN - 3 : LOGN; }
+
+// Twiddles of thread b's round that starts at forward level LVL, where each
+// thread has one set in it (otherwise the round loads them itself).
+template <int LOGN, int LVL>
+__device__ __forceinline__ void fwd_next_twiddles(uint2 (&w)[7], const Limb &T, uint32_t b) {
+  constexpr int LEFT = middle_end<LOGN>() - LVL;
+  if constexpr (LEFT > 0) {
+    if constexpr (middle_levels<LEFT>() == 3) {
+      uint32_t i, o;
+      set_of<3, ((1u << LOGN) >> (LVL + 3)), (1u << LOGN)>(b, i, o);
+      fwd_twiddles<3, 1u << LVL>(w, T.fw, i);
+    }
+  } else if constexpr (LOGN >= 6) {
+    thread_twiddles(w, T.fw_last + 8 * b, true);
+  }
+}
+
+// The same for the inverse round at level G.
+template <int LOGN, int G>
+__device__ __forceinline__ void inv_next_twiddles(uint2 (&w)[7], const Limb &T, uint32_t b) {
+  constexpr int LEFT = middle_end<LOGN>() - G;
+  if constexpr (LEFT > 0) {
+    if constexpr (middle_levels<LEFT>() == 3) {
+      uint32_t i, o;
+      set_of<3, (1u << G), (1u << LOGN)>(b, i, o);
+      inv_twiddles<3, (1u << LOGN) / (2u << G)>(w, T.iv, i);
+    }
+  }
+}
+
 template <int LOGN, int R, int LVL, int P>
-__device__ __forceinline__ void fwd_middle(uint32_t *const (&buf)[P], const Limb &T, uint32_t b) {
+__device__ __forceinline__ void fwd_middle(uint32_t *const (&buf)[P], uint2 (&w)[7], const Limb &T, uint32_t b) {
   constexpr uint32_t N = 1u << LOGN, S = N >> 3, M0 = 1u << LVL, U = N >> (LVL + R);
 #pragma unroll
   for (uint32_t t = 0; t < (N >> R) / S; ++t) {
     uint32_t i, o;
     set_of<R, U, N>(b + t * S, i, o);
     const uint32_t base = pad((i << R) * U + o);
-    uint2 w[7];
-    fwd_twiddles<R, M0>(w, T.fw, i);
+    if constexpr (R < 3) fwd_twiddles<R, M0>(w, T.fw, i);
     uint32_t v[P][8];
 #pragma unroll
     for (int p = 0; p < P; ++p)
 #pragma unroll
       for (uint32_t k = 0; k < (1u << R); ++k) v[p][k] = buf[p][base + pad(k * U)];
-    fwd_levels<R, LVL, P>(v, w, T.q);
+    fwd_levels<R, LVL, P>(v, w, T);
 #pragma unroll
     for (int p = 0; p < P; ++p)
 #pragma unroll
@@ -306,15 +342,14 @@ __device__ __forceinline__ void fwd_middle(uint32_t *const (&buf)[P], const Limb
 }
 
 template <int LOGN, int R, int G>
-__device__ __forceinline__ void inv_middle(uint32_t *buf, const Limb &T, uint32_t b) {
+__device__ __forceinline__ void inv_middle(uint32_t *buf, uint2 (&w)[7], const Limb &T, uint32_t b) {
   constexpr uint32_t N = 1u << LOGN, S = N >> 3, T0 = 1u << G;
 #pragma unroll
   for (uint32_t t = 0; t < (N >> R) / S; ++t) {
     uint32_t i, o;
     set_of<R, T0, N>(b + t * S, i, o);
     uint32_t *p = buf + pad((i << R) * T0 + o);
-    uint2 w[7];
-    inv_twiddles<R, N / (2 * T0)>(w, T.iv, i);
+    if constexpr (R < 3) inv_twiddles<R, N / (2 * T0)>(w, T.iv, i);
     uint32_t v[1][8];
 #pragma unroll
     for (uint32_t k = 0; k < (1u << R); ++k) v[0][k] = p[pad(k * T0)];
@@ -324,25 +359,32 @@ __device__ __forceinline__ void inv_middle(uint32_t *buf, const Limb &T, uint32_
   }
 }
 
+// The rounds from level LVL (G) to the bit-reversed (last) one; w holds the
+// first one's twiddles on entry and the next round's on return.
 template <int LOGN, int LVL, int P>
-__device__ __forceinline__ void fwd_middles(uint32_t *const (&buf)[P], const Limb &T, uint32_t b, bool act) {
-  constexpr int END = LOGN >= 6 ? LOGN - 3 : LOGN;
-  if constexpr (LVL < END) {
-    constexpr int R = middle_levels<END - LVL>();
-    if (act) fwd_middle<LOGN, R, LVL, P>(buf, T, b);
+__device__ __forceinline__ void fwd_middles(uint32_t *const (&buf)[P], uint2 (&w)[7], const Limb &T, uint32_t b,
+                                            bool act) {
+  if constexpr (LVL < middle_end<LOGN>()) {
+    constexpr int R = middle_levels<middle_end<LOGN>() - LVL>();
+    if (act) {
+      fwd_middle<LOGN, R, LVL, P>(buf, w, T, b);
+      fwd_next_twiddles<LOGN, LVL + R>(w, T, b);
+    }
     __syncthreads();
-    fwd_middles<LOGN, LVL + R, P>(buf, T, b, act);
+    fwd_middles<LOGN, LVL + R, P>(buf, w, T, b, act);
   }
 }
 
 template <int LOGN, int G>
-__device__ __forceinline__ void inv_middles(uint32_t *buf, const Limb &T, uint32_t b, bool act) {
-  constexpr int END = LOGN >= 6 ? LOGN - 3 : LOGN;
-  if constexpr (G < END) {
-    constexpr int R = middle_levels<END - G>();
-    if (act) inv_middle<LOGN, R, G>(buf, T, b);
+__device__ __forceinline__ void inv_middles(uint32_t *buf, uint2 (&w)[7], const Limb &T, uint32_t b, bool act) {
+  if constexpr (G < middle_end<LOGN>()) {
+    constexpr int R = middle_levels<middle_end<LOGN>() - G>();
+    if (act) {
+      inv_middle<LOGN, R, G>(buf, w, T, b);
+      inv_next_twiddles<LOGN, G + R>(w, T, b);
+    }
     __syncthreads();
-    inv_middles<LOGN, G + R>(buf, T, b, act);
+    inv_middles<LOGN, G + R>(buf, w, T, b, act);
   }
 }
 
@@ -356,24 +398,23 @@ template <int LOGN, int P>
 __device__ __forceinline__ void forward(uint32_t (&v)[P][8], uint32_t *const (&buf)[P], const Limb &T, uint32_t b,
                                         bool act) {
   constexpr uint32_t N = 1u << LOGN, S = N >> 3;
+  uint2 w[7];
   if (act) {
-    uint2 w[7];
 #pragma unroll
     for (int k = 0; k < 7; ++k) w[k] = T.fw8[k + 1];
-    fwd_levels<3, 0, P>(v, w, T.q);
+    fwd_levels<3, 0, P>(v, w, T);
     const uint32_t base = pad(b);
 #pragma unroll
     for (int p = 0; p < P; ++p)
 #pragma unroll
       for (uint32_t k = 0; k < 8; ++k) buf[p][base + pad(k * S)] = v[p][k];
+    fwd_next_twiddles<LOGN, 3>(w, T, b);
   }
   __syncthreads();
-  fwd_middles<LOGN, 3, P>(buf, T, b, act);
+  fwd_middles<LOGN, 3, P>(buf, w, T, b, act);
   if (!act) return;
   if constexpr (LOGN >= 6) {
     const uint32_t base = pad(8 * brev(b, LOGN - 3));
-    uint2 w[7];
-    thread_twiddles(w, T.fw_last + 8 * b, true);
 #pragma unroll
     for (int p = 0; p < P; ++p) {
       const uint4 x = *reinterpret_cast<const uint4 *>(buf[p] + base);
@@ -381,7 +422,7 @@ __device__ __forceinline__ void forward(uint32_t (&v)[P][8], uint32_t *const (&b
       v[p][0] = x.x, v[p][1] = x.y, v[p][2] = x.z, v[p][3] = x.w;
       v[p][4] = y.x, v[p][5] = y.y, v[p][6] = y.z, v[p][7] = y.w;
     }
-    fwd_levels<3, LOGN - 3, P>(v, w, T.q);
+    fwd_levels<3, LOGN - 3, P>(v, w, T);
 #pragma unroll
     for (int p = 0; p < P; ++p) {
       // position 8i + k holds slot (N/8) brv3(k) + b
@@ -397,28 +438,35 @@ __device__ __forceinline__ void forward(uint32_t (&v)[P][8], uint32_t *const (&b
   }
 }
 
-// Inverse NTT of one polynomial of one limb. In: v[e] = slot b + (N/8) e,
-// values < 2q. Out: v[k] = coefficient b + (N/8) k, below q. After its last
-// barrier a thread reads only the positions b + (N/8) k of the buffer.
+// Twiddles of the first inverse round, which a kernel loads before it has the
+// values.
 template <int LOGN>
-__device__ __forceinline__ void inverse(uint32_t (&v)[1][8], uint32_t *buf, const Limb &T, uint32_t b, bool act) {
+__device__ __forceinline__ void inv_first_twiddles(uint2 (&w)[7], const Limb &T, uint32_t b) {
+  if constexpr (LOGN >= 6) thread_twiddles(w, T.iv_first + 8 * b, false);
+  else inv_twiddles<3, (1u << LOGN) / 2>(w, T.iv, brev(b, LOGN - 3));
+}
+
+// Inverse NTT of one polynomial of one limb. In: v[e] = slot b + (N/8) e,
+// values < 2q, and w from inv_first_twiddles. Out: v[k] = coefficient
+// b + (N/8) k, below q. After its last barrier a thread reads only the
+// positions b + (N/8) k of the buffer.
+template <int LOGN>
+__device__ __forceinline__ void inverse(uint32_t (&v)[1][8], uint32_t *buf, uint2 (&w)[7], const Limb &T,
+                                        uint32_t b, bool act) {
   constexpr uint32_t N = 1u << LOGN, S = N >> 3;
-  uint2 w[7];
   if (act) {
-    const uint32_t i = brev(b, LOGN - 3);
-    if constexpr (LOGN >= 6) thread_twiddles(w, T.iv_first + 8 * b, false);
-    else inv_twiddles<3, (N >> 1)>(w, T.iv, i);
-    // position 8i + k holds slot (N/8) brv3(k) + b
+    // position 8i + k, i = brv(b), holds slot (N/8) brv3(k) + b
     const uint32_t t1 = v[0][1], t3 = v[0][3];
     v[0][1] = v[0][4], v[0][4] = t1;
     v[0][3] = v[0][6], v[0][6] = t3;
     inv_levels<3, false, 1>(v, w, T);
-    uint4 *p = reinterpret_cast<uint4 *>(buf + pad(8 * i));
+    uint4 *p = reinterpret_cast<uint4 *>(buf + pad(8 * brev(b, LOGN - 3)));
     p[0] = make_uint4(v[0][0], v[0][1], v[0][2], v[0][3]);
     p[1] = make_uint4(v[0][4], v[0][5], v[0][6], v[0][7]);
+    inv_next_twiddles<LOGN, 3>(w, T, b);
   }
   __syncthreads();
-  inv_middles<LOGN, 3>(buf, T, b, act);
+  inv_middles<LOGN, 3>(buf, w, T, b, act);
   if (!act) return;
   const uint32_t base = pad(b);
 #pragma unroll
@@ -444,18 +492,13 @@ __device__ __forceinline__ void dcp_digits(const Ring &R, const Limb &T, uint32_
                                            uint32_t (&d)[digits<L>()]) {
   uint64_t x = r0;
   if constexpr (L > 1) {
-    const uint32_t q1 = R.limb[1].q;
-    const uint32_t k = shoup(r1 + R.crt_add - r0, R.q0_inv, q1);
+    const uint32_t k = shoup(r1 + R.crt_add - r0, R.q0_inv, R.limb[1].q);
     x += (uint64_t)R.limb[0].q * k;
   }
   const uint64_t y = x + (x > R.half_Q ? R.off_neg : R.off_pos);
 #pragma unroll
   for (int i = 0; i < digits<L>(); ++i)
     d[i] = ((uint32_t)((int64_t)y >> (LOG_BASE * i)) & R.digit_mask[i]) + T.digit_add[i];
-}
-
-__device__ __forceinline__ void prefetch_l1(const void *p) {
-  asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
 }
 
 // Thread-block cluster helpers: the CTAs of a tree node hand each other
@@ -478,6 +521,10 @@ __device__ __forceinline__ void st_peer(uint32_t addr, uint32_t v) {
 }
 __device__ __forceinline__ void cluster_arrive() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+// No memory ordering: for a CTA that is done reading its own shared memory.
+__device__ __forceinline__ void cluster_arrive_relaxed() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");

@@ -142,6 +142,7 @@ static int ring_tables_impl(const gpir_params_t *params, ntt::Ring *out) {
     T.n_inv = shoup_pair(ninv);
     T.r32 = shoup_pair((1ull << 32) % q);
     T.q = (uint32_t)q;
+    T.q2 = (uint32_t)(2 * q);
     T.one_s = shoup_quotient(1, q);
   }
   if (L == 2) {
