@@ -148,6 +148,7 @@ constexpr int T_MAX_JOBS = 8;
 struct TmJob {
   CUtensorMap ct_map;                   // box (8 slots, 1, 2, 64 k, BOX_CLIENTS clients)
   uint32_t M, d1, mblk, nblk, kch, upe;
+  uint32_t reads;                       // ring tiles read from an entry: units x k-chunks
   TmDiv mblk_d, nblk_d, kch_d, upe_d;   // the same four as divisors
   uint64_t entry0, unit0, task0;        // first entry / unit / ingest task of the job
   const uint16_t *b_tiles;              // [slot][nblk][kch] x 24 KB
@@ -162,7 +163,7 @@ struct TmemParams {
   uint32_t hints;                       // 1: raw boxes evict-first, ring stores evict-last in L2
   uint64_t n_entries, n_units, n_tasks; // over all jobs
   uint8_t *ring;                        // [R][8 slots][kch_max] x 8 KB
-  uint32_t *ready, *consumed;           // [n_entries] each: tasks ingested, units that read the entry
+  uint32_t *ready, *consumed;           // [n_entries] each: tasks ingested, ring tiles read
   unsigned long long *ctr;              // [0] next unit, [1] next ingest task
   unsigned int *err;
   unsigned long long *prof;             // wait-cycle counters (traced instantiation only)
@@ -259,11 +260,12 @@ __device__ __forceinline__ void tmem_ld4x3(uint32_t t0, uint32_t t1, uint32_t t2
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%12];\n"
       "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%13];\n"
-      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%8,%9,%10,%11}, [%14];"
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%8,%9,%10,%11}, [%14];\n"
+      "tcgen05.wait::ld.sync.aligned;"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11])
-      : "r"(t0), "r"(t1), "r"(t2));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      : "r"(t0), "r"(t1), "r"(t2)
+      : "memory");
 }
 
 // Ring encoding of a ciphertext residue x < q: the four 7-bit fields of
@@ -370,7 +372,7 @@ __global__ void tm_pack_db_kernel(const Pack12Params p, uint64_t total) {
 // ring and for claims already made), with one ready and one consumed counter
 // per entry (entries of different jobs need different counts); ring entries
 // are strided by the largest job's k-chunk count. The ring holds encoded raw
-// residues and an entry is released as soon as its units' last k-chunks have
+// residues and an entry is released as soon as every k-chunk of its units has
 // landed in shared memory. SM-pair form (PAIR, one job): a pair unit covers
 // entries 2 E2 (even CTA) and 2 E2 + 1 (odd CTA) against one database tile;
 // each CTA copies its own ring tile and its half of B and converts its own A
@@ -399,8 +401,7 @@ __global__ void __launch_bounds__(T_THREADS, 1) tc_tmem_kernel(const __grid_cons
   uint64_t *ostage_empty = ostage_full + 1;
   uint64_t *stage_unit = ostage_empty + 1;        // [NS] unit of the B stage
   uint64_t *slot_unit = stage_unit + NS;          // [RS] unit of the ring slot
-  uint64_t *slot_kc = slot_unit + RS;             // [RS] k-chunk of the unit in the ring slot
-  uint64_t *acc_unit = slot_kc + RS;              // [2]
+  uint64_t *acc_unit = slot_unit + RS;            // [2]
   uint64_t *task_slot = acc_unit + 2;
   uint64_t *ostage_unit = task_slot + 1;
   uint64_t *mail = ostage_unit + 1;               // pair: [4] claimed units, even -> odd CTA
@@ -411,7 +412,7 @@ __global__ void __launch_bounds__(T_THREADS, 1) tc_tmem_kernel(const __grid_cons
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(task_ok + 1);
   volatile uint32_t *abort_flag = tmem_slot + 1;
   // barriers and tags above, in 8-byte words, within the 1 KB reserved for them
-  static_assert(8 * (3 * NS + 4 * RS + 2 * T_ABUF_MAX + 4 + 4 + 2 + 2 + 12 + 2 + 1 + 1) <= 1024,
+  static_assert(8 * (3 * NS + 3 * RS + 2 * T_ABUF_MAX + 4 + 4 + 2 + 2 + 12 + 2 + 1 + 1) <= 1024,
                 "tensor-memory kernel barrier area exceeds its reservation");
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -612,7 +613,6 @@ __global__ void __launch_bounds__(T_THREADS, 1) tc_tmem_kernel(const __grid_cons
         for (uint32_t kc = 0; kc < kch; ++kc) {
           if (!(ok = TM_TIMED(kTPWaitEmpty, wait(&rempty[r], rph ^ 1u, kErrTmaWait)))) break;
           slot_unit[r] = u;
-          slot_kc[r] = kc;
           mbar_arrive_expect_tx(&rfull[r], T_RAW_TILE);
           bulk_g2s(rslots + r * T_RAW_TILE, src_a + (uint64_t)kc * T_RAW_TILE, T_RAW_TILE, &rfull[r]);
           r_issued |= 1u << r;
@@ -698,9 +698,10 @@ __global__ void __launch_bounds__(T_THREADS, 1) tc_tmem_kernel(const __grid_cons
         }
         break;
       }
-      // the unit's last ring tile is in shared memory: its ring entry may be reused
-      if (qw == 0 && lane == 0 && slot_kc[r] + 1 == p.job[job_of_unit<MULTI>(p, un)].kch)
-        atomicAdd(&p.consumed[entry_of(un)], 1u);
+      // this ring tile is in shared memory. Every k-chunk is counted: copies
+      // complete in any order, so the last one's landing does not tell that
+      // the others have read their part of the entry.
+      if (qw == 0 && lane == 0) atomicAdd(&p.consumed[entry_of(un)], 1u);
       // this thread's digit plane: 8 bytes per k octet (conflict-free: the
       // warp's 32 reads of a step cover every bank twice)
       const uint2 *row = reinterpret_cast<const uint2 *>(rslots + r * T_RAW_TILE) + m * 32;
@@ -713,10 +714,6 @@ __global__ void __launch_bounds__(T_THREADS, 1) tc_tmem_kernel(const __grid_cons
         wv[4 * j + 2] = plane_pair(z.y, 0x5140u);
         wv[4 * j + 3] = plane_pair(z.y, 0x5342u);
       }
-      // the digits are in registers (every loaded word went into them): the
-      // ring slot may be refilled
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&rempty[r]);
       const uint64_t tst = PROF ? clock64() : 0;
       if (conv_counter) pc[PROF ? kTCBusy : 0] += tst - tconv;
       // the A buffer's previous k-chunk must have been read by its MMAs before
@@ -730,6 +727,9 @@ __global__ void __launch_bounds__(T_THREADS, 1) tc_tmem_kernel(const __grid_cons
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
+        // the ring slot may be refilled: the store has consumed every word
+        // read from it (after the reads alone some may still be in flight)
+        mbar_arrive(&rempty[r]);
         if (PAIR && rank != 0)
           mbar_arrive_remote_relaxed(map_peer(smem_u32(&afull[ab]), 0));
         else
@@ -1068,7 +1068,7 @@ __global__ void __launch_bounds__(T_THREADS, 1) tc_tmem_kernel(const __grid_cons
                           TM_TIMED(kTIWaitSlot, wait_claims(first_unit_of(E - p.lookahead)));
         const bool free =
             near && (E < p.R || TM_TIMED(kTIWaitSlot, wait_count(&p.consumed[E - p.R],
-                                                                 p.job[job_of_entry<MULTI>(p, E - p.R)].upe)));
+                                                                 p.job[job_of_entry<MULTI>(p, E - p.R)].reads)));
         *task_ok = free ? 1u : 0u;   // task_slot may still be read for this task
       }
       asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
@@ -1331,6 +1331,7 @@ int tc_launch_tmem_jobs(const gpir_job_t *jobs, uint32_t njobs, size_t ring_targ
     jb.nblk = (db->d1 + T_NCOLS - 1) / T_NCOLS;
     jb.kch = (db->d0 + T_KCHUNK - 1) / T_KCHUNK;
     jb.upe = tp.spg * jb.nblk;
+    jb.reads = jb.upe * jb.kch;
     jb.mblk_d = tm_div(jb.mblk);
     jb.nblk_d = tm_div(jb.nblk);
     jb.kch_d = tm_div(jb.kch);
