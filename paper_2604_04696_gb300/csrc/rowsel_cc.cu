@@ -52,7 +52,10 @@ __global__ void __launch_bounds__(C::THREADS, C::MINB)
     rowsel_cc_kernel(const __grid_constant__ CUtensorMap ct_map, const __grid_constant__ CUtensorMap db_map,
                      uint32_t *__restrict__ out, const CcParams p) {
   extern __shared__ __align__(128) uint8_t smem_raw[];
-  uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
+  // aligned by an offset, so that it stays a shared-memory pointer to the
+  // compiler: through a rounded integer address every read was a generic load
+  // (32 clients, 256x64: 1.42 -> 1.31 ms; 8 clients 0.411 -> 0.378 ms)
+  uint8_t *smem = smem_raw + ((0u - smem_u32(smem_raw)) & 127u);
   uint32_t *ct_s = reinterpret_cast<uint32_t *>(smem);
   uint32_t *db_s = ct_s + C::STAGES * C::CT_WORDS;
   uint64_t *full = reinterpret_cast<uint64_t *>(db_s + C::STAGES * C::DB_WORDS);
