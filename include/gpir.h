@@ -140,8 +140,8 @@ int gpir_rowsel_batch_host(const gpir_db_t *db, uint32_t batch, const uint32_t *
  * per 8 jobs (databases uploaded without that kernel's digit tiles: the
  * two-pass kernels). CUDA-core and IMMA paths use one launch per job.
  * GPIR_PATH_AUTO runs each job on the path gpir_rowsel_batch would choose for
- * its batch (the autotuned one, else tensor cores from batch 8), the
- * tensor-core jobs together. All jobs must share the same params (N, L,
+ * its batch (the autotuned one, else the static rule of gpir_selected_path), the
+ * tensor-core jobs together (those of up to 8 clients in the streaming kernel). All jobs must share the same params (N, L,
  * primes) and every job's
  * ct / out must not overlap any other buffer of the call. The tensor-core
  * workspace for the call is grown on demand (not while the stream is being
@@ -222,7 +222,9 @@ long gpir_set_fail_alloc(long n);
  * shape (-1 if none chosen yet). Host-only. */
 int gpir_num_variants(int path);
 /* The path GPIR_PATH_AUTO resolves to for `batch` clients (tuned, else the
- * static rule: tensor cores from 8 clients up when prepared). Host-only. */
+ * static rule when prepared: tensor cores from 8 clients up, and below that from
+ * 2 clients on databases of more than 192 rows, from 5 on smaller ones, if the
+ * database has enough 8-slot x 32-column tiles for the SMs). Host-only. */
 int gpir_selected_path(const gpir_db_t *db, uint32_t batch);
 int gpir_selected_variant(const gpir_db_t *db, uint32_t batch, int path);
 /* Force a variant for (path, batch, D0, D1) of this database (testing). */

@@ -223,14 +223,20 @@ int pick_variant(const gpir_db *db, uint32_t batch, int path) {
   switch (path) {
     case GPIR_PATH_CUDACORE: return rowsel_cc_default_variant(batch, db->d0, db->d1);
     case GPIR_PATH_IMMA: return rowsel_imma_default_variant(batch, db->d0, db->d1);
-    case GPIR_PATH_TC: return rowsel_tc_default_variant(batch, db->d0, db->d1);
+    case GPIR_PATH_TC: return rowsel_tc_default_variant(db, batch);
   }
   return -1;
 }
 
 // GPIR_PATH_AUTO: the path the autotuner measured fastest for this batch size,
-// else a static choice: tensor cores once a batch fills a 32-row tile well
-// (batch >= 8), CUDA cores below that (one client wastes 15/16 of an MMA tile).
+// else a static choice. Where the streaming kernel applies (up to 8 clients):
+// tensor cores from 2 clients on databases of more than 192 rows, from 5 on
+// smaller ones, whose units are too short to hide its pipeline's ends. N = 4096,
+// 2 limbs, us on the CUDA cores / streaming: 2 clients 211 / 131 and 3 clients
+// 213 / 132 (256x64), 4 clients 237 / 166 (600x8) and 244 / 202 (300x33), but 35 / 47
+// (64x32) and 49 / 55 (100x16); 8 clients 68 / 55 and 84 / 59 on those two; one
+// client 94 / 129 (256x64). Elsewhere: tensor cores from 8 clients (one client
+// wastes 15/16 of an MMA tile).
 int resolve_path(const gpir_db *db, int path, uint32_t batch) {
   if (path == GPIR_PATH_AUTO) {
     {
@@ -239,7 +245,8 @@ int resolve_path(const gpir_db *db, int path, uint32_t batch) {
       if (it != db->variants->end()) return it->second;
     }
     const bool tc = db->path_mask & GPIR_PATH_TC, cc = db->path_mask & GPIR_PATH_CUDACORE;
-    if (tc && (batch >= 8 || !cc)) return GPIR_PATH_TC;
+    const uint32_t from = !rowsel_stream_preferred(db, batch) ? 8u : db->d0 > 192 ? 2u : 5u;
+    if (tc && (batch >= from || !cc)) return GPIR_PATH_TC;
     if (cc) return GPIR_PATH_CUDACORE;
     if (db->path_mask & GPIR_PATH_IMMA) return GPIR_PATH_IMMA;
     return -1;
@@ -377,6 +384,7 @@ int gpir_db_upload(const gpir_params_t *params, uint32_t d0, uint32_t d1, const 
   if (path_mask & GPIR_PATH_TC) {
     rc = rowsel_tc_prepare(db, s);
     if (rc == GPIR_OK) rc = rowsel_tmem_prepare(db, s);
+    if (rc == GPIR_OK) rc = rowsel_stream_prepare(db, s);
     if (rc != GPIR_OK) goto fail;
   }
   *out = db;
@@ -391,6 +399,8 @@ int gpir_db_free(gpir_db_t *db) {
   if (db->db_pmajor) cudaFree(db->db_pmajor);
   if (db->db_digits) cudaFree(db->db_digits);
   if (db->db_digits12) cudaFree(db->db_digits12);
+  if (db->db_fields) cudaFree(db->db_fields);
+  if (db->db_corr) cudaFree(db->db_corr);
   if (db->ws_ct) cudaFree(db->ws_ct);
   if (db->ws_out) cudaFree(db->ws_out);
   delete db->variants;
@@ -402,7 +412,7 @@ int gpir_db_free(gpir_db_t *db) {
 size_t gpir_db_device_bytes(const gpir_db_t *db) {
   if (!db) return 0;
   size_t b = (size_t)db->d0 * db->d1 * db->params.num_limbs * db->params.n * 4;
-  return b + db->db_digits_bytes + db->db_digits12_bytes;
+  return b + db->db_digits_bytes + db->db_digits12_bytes + db->db_fields_bytes + db->db_corr_bytes;
 }
 
 int gpir_rowsel_batch(const gpir_db_t *db, uint32_t batch, const uint32_t *ct_dev, uint32_t *out_dev, int path,

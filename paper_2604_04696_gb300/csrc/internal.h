@@ -54,6 +54,11 @@ struct gpir_db {
   size_t db_digits_bytes;
   uint16_t *db_digits12;
   size_t db_digits12_bytes;
+  // and the four 7-bit fields of the residues with the columns' corrections (rowsel_stream.cu).
+  uint8_t *db_fields;
+  size_t db_fields_bytes;
+  uint32_t *db_corr;
+  size_t db_corr_bytes;
   // Host-buffer entry point workspace.
   uint32_t *ws_ct, *ws_out;
   size_t ws_ct_bytes, ws_out_bytes;
@@ -112,7 +117,7 @@ int rowsel_tc_prepare(gpir_db *db, cudaStream_t stream);
 int rowsel_tc_launch(const gpir_db *db, uint32_t batch, const uint32_t *ct, uint32_t *out,
                      int variant, cudaStream_t stream);
 int rowsel_tc_num_variants();
-int rowsel_tc_default_variant(uint32_t batch, uint32_t d0, uint32_t d1);
+int rowsel_tc_default_variant(const gpir_db *db, uint32_t batch);
 
 // Tracing hooks: trace_begin returns -1 (and records nothing) when disabled.
 int trace_begin(const char *name, cudaStream_t s);
@@ -125,12 +130,19 @@ void trace_counters(const unsigned long long *dev, int n, cudaStream_t s);
 // and one launch (pair: the SM-pair form; GPIR_ENOTSUP if it does not apply).
 int rowsel_tmem_prepare(gpir_db *db, cudaStream_t stream);
 // the path gpir_rowsel_batch runs for (db, batch) under `path` (GPIR_PATH_AUTO:
-// the autotuned one, else tensor cores from batch 8, CUDA cores below); < 0: none
+// the autotuned one, else the static rule of gpir_abi.cu); < 0: none
 int resolve_path(const gpir_db *db, int path, uint32_t batch);
 // several RowSel jobs (one parameter set) in tensor-memory kernel launches of up to 8 jobs each
 int rowsel_tmem_multi(const gpir_job_t *jobs, uint32_t njobs, cudaStream_t stream);
 int tc_launch_tmem(const gpir_db *db, uint32_t batch, const uint32_t *ct, uint32_t *out, size_t ring_target,
                    uint32_t lookahead_mb, uint32_t hints, bool pair, cudaStream_t stream);
+// Streaming kernel (rowsel_stream.cu): its database layout, built at upload, and
+// launches of up to 8 jobs of one parameter set each.
+int rowsel_stream_prepare(gpir_db *db, cudaStream_t stream);
+int rowsel_stream_launch(const gpir_job_t *jobs, uint32_t njobs, cudaStream_t stream);
+constexpr int kTcVariantStream = 12;   // its tile variant
+// whether untuned batches of this database take it on the tensor-core path
+bool rowsel_stream_preferred(const gpir_db *db, uint32_t batch);
 // The tensor-core workspace kept for (current device, stream), grown on demand
 // (never inside a stream capture: GPIR_ENOMEM then).
 int tc_stream_workspace(cudaStream_t stream, size_t need, uint8_t **out);

@@ -3,9 +3,8 @@
 // job list), and CUDA-graph plans of such calls.
 //
 // Tensor-core path: one job runs the kernel tuned for its batch; several jobs
-// have their entries, work units and ingest tasks numbered into one index
-// space and run in ONE persistent launch of the tensor-memory kernel, up to 8
-// jobs per launch. CUDA-core and IMMA paths: one launch per job.
+// run up to 8 per persistent launch, their work numbered into one index space:
+// small batches in the streaming kernel, the others in the tensor-memory kernel. CUDA-core and IMMA paths: one launch per job.
 // GPIR_PATH_AUTO: each job on the path gpir_rowsel_batch would choose for it.
 #include <cuda_runtime.h>
 #include <string.h>
@@ -17,16 +16,31 @@
 
 namespace gpir {
 
-// Tensor-core jobs of one call: one job runs the kernel tuned for its batch;
-// several run in one persistent tensor-memory launch per 8 jobs (databases
+// Tensor-core jobs of one call: one job runs the kernel tuned for its batch. Of
+// several, those whose variant is the streaming kernel run in its launches of 8
+// jobs, the others in one persistent tensor-memory launch per 8 jobs (databases
 // uploaded without its digit tiles: the two-pass kernels).
 static int tc_jobs(const gpir_job_t *jobs, uint32_t njobs, cudaStream_t stream) {
   if (njobs == 1)
     return dispatch(jobs[0].db, jobs[0].batch, jobs[0].ct, jobs[0].out, GPIR_PATH_TC,
                     pick_variant(jobs[0].db, jobs[0].batch, GPIR_PATH_TC), stream);
+  std::vector<gpir_job_t> part[2];   // tensor-memory, streaming
+  try {
+    part[0].reserve(njobs);
+    part[1].reserve(njobs);
+  } catch (...) {   // no exception crosses the C ABI
+    return GPIR_ENOMEM;
+  }
+  for (uint32_t k = 0; k < njobs; ++k)
+    part[pick_variant(jobs[k].db, jobs[k].batch, GPIR_PATH_TC) == kTcVariantStream].push_back(jobs[k]);
+  if (!part[1].empty()) {
+    const int rc = rowsel_stream_launch(part[1].data(), (uint32_t)part[1].size(), stream);
+    if (rc != GPIR_OK || part[0].empty()) return rc;
+  }
   bool tmem = true;
-  for (uint32_t k = 0; k < njobs; ++k) tmem = tmem && jobs[k].db->db_digits12 != nullptr;
-  return tmem ? rowsel_tmem_multi(jobs, njobs, stream) : rowsel_tc_multi(jobs, njobs, stream);
+  for (const gpir_job_t &j : part[0]) tmem = tmem && j.db->db_digits12 != nullptr;
+  return tmem ? rowsel_tmem_multi(part[0].data(), (uint32_t)part[0].size(), stream)
+              : rowsel_tc_multi(part[0].data(), (uint32_t)part[0].size(), stream);
 }
 
 int rowsel_multi_launch(const gpir_job_t *jobs, uint32_t njobs, int path, cudaStream_t stream) {

@@ -1725,9 +1725,12 @@ static TcLimb make_limb(uint32_t q) {
 
 }  // namespace
 
-// Untuned batches: the tensor-memory kernel, single CTA (variant 8), which
-// the autotuner picks from batch 8 up on every database shape measured.
-int rowsel_tc_default_variant(uint32_t, uint32_t, uint32_t) { return 8; }
+// Untuned batches: the streaming kernel for one block of 16 rows (see
+// rowsel_stream_preferred), above it the tensor-memory kernel, single CTA
+// (variant 8), which the autotuner picks there on every database shape measured.
+int rowsel_tc_default_variant(const gpir_db *db, uint32_t batch) {
+  return rowsel_stream_preferred(db, batch) ? kTcVariantStream : 8;
+}
 
 int rowsel_tc_prepare(gpir_db *db, cudaStream_t stream) {
   const uint32_t L = db->params.num_limbs, N = db->params.n;
@@ -1938,6 +1941,7 @@ enum TcKernelKind : uint32_t {
   kKindPair = 3,
   kKindTmem = 4,       // rowsel_tmem.cu: A in tensor memory, 12 digit products
   kKindTmemPair = 5,   // its SM-pair form
+  kKindStream = 6,     // rowsel_stream.cu: the database streamed through tensor memory
 };
 struct FusedVariant {
   uint32_t kind;           // TcKernelKind
@@ -1959,6 +1963,7 @@ constexpr FusedVariant kFusedVariants[] = {
     {kKindTmemPair, 48, 0, 16},         // 9: its SM-pair form
     {kKindTmem, 24, 1, 8},              // 10: 8 with raw boxes evict-first, ring stores evict-last
     {kKindTmemPair, 48, 1, 16},         // 11: 9 with those hints
+    {kKindStream, 0, 0, 0},             // 12: the database streamed through tensor memory
 };
 constexpr int kNumTcVariants = (int)(sizeof(kFusedVariants) / sizeof(kFusedVariants[0]));
 
@@ -2226,6 +2231,15 @@ int rowsel_tc_launch(const gpir_db *db, uint32_t batch, const uint32_t *ct, uint
     job.ct = ct;
     job.out = out;
     return rowsel_tc_multi(&job, 1, stream);   // two-pass: ingest to HBM, then GEMM
+  }
+  if (v.kind == kKindStream) {
+    gpir_job_t job;
+    memset(&job, 0, sizeof(job));
+    job.db = db;
+    job.batch = batch;
+    job.ct = ct;
+    job.out = out;
+    return rowsel_stream_launch(&job, 1, stream);
   }
   if (v.kind == kKindTmem || v.kind == kKindTmemPair) {
     const bool pr = v.kind == kKindTmemPair;
