@@ -42,8 +42,8 @@
 //     only B from shared memory;
 //   - one elected lane issues tcgen05.mma .kind::f16 with A in tensor memory
 //     (M = 128 or 256, N = 192, K = 16);
-//   - epilogue warps drain the double-buffered accumulators and a store warp
-//     writes the p-major output.
+//   - epilogue warps drain the double-buffered accumulators and the store warps
+//     write the p-major output.
 // Tensor memory (512 columns): accumulators at [0, 192) and [192, 384), and
 // 128 columns of A buffers at 384: four buffers of one k-chunk (64 k of fp16
 // pairs, 32 columns) or two of two consecutive k-chunks (64 columns, one
@@ -80,7 +80,7 @@ constexpr int32_t kOffB = 512 * (1 + (1 << 10));
 
 // Warp roles (896 threads). Tensor-memory lane quarter of a warp = warp % 4.
 constexpr int W_PROD = 0, W_MMA = 1, W_STORE = 2;
-constexpr int W_RELAY = 3;                           // SM pair: hands finished groups to the odd CTA
+constexpr int W_RELAY = 3;                           // SM pair: hands finished groups to the odd CTA; else a second store warp
 constexpr int W_CONV0 = 4, N_CONV = 8;               // two converter sets of 4 warps (quarters 0..3),
                                                      // set s converts stages s and s + 2
 constexpr int W_EPI0 = 12, N_EPI = 8;                // 8 epilogue warps: quarter, column half
@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(T_THREADS, 1) tc_tmem_kernel(const __grid_cons
     mbar_init(&box_bar[0], 1);
     mbar_init(&box_bar[1], 1);
     mbar_init(ostage_full, N_EPI);
-    mbar_init(ostage_empty, 1);
+    mbar_init(ostage_empty, PAIR ? 1 : 2);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -979,8 +979,17 @@ __global__ void __launch_bounds__(T_THREADS, 1) tc_tmem_kernel(const __grid_cons
         hb ^= 1u;
       }
     }
-  } else if (warp == W_STORE) {
-    // ---------------- output store warp ----------------
+  } else if (warp == W_STORE || (!PAIR && warp == W_RELAY)) {
+    // ---------------- output store warps (one in the pair form, else two) ----------------
+    // A store writes 32 words of 32 sectors. At few database rows (one group per
+    // unit) the output bounds the kernel: one warp, a load and a store in turn,
+    // was busy 83% of the time at 256 rows and 32 clients while the MMAs waited
+    // for accumulators. Two warps, and four rows read from the stage before any
+    // is written so that a warp's stores follow one another: 256x64, 2 limbs of
+    // 4096 slots, 32 clients 541 -> 501 us, 128 clients 2112 -> 1865 us.
+    constexpr uint32_t NST = PAIR ? 1 : 2, NROW = 4;
+    static_assert(T_MROWS % (NROW * NST) == 0, "whole steps of rows");
+    const uint32_t stage_s = smem_u32(out_stage);
     uint32_t ph = 0;
     for (;;) {
       if (!__all_sync(0xffffffffu, wait(ostage_full, ph, kErrMmaWait))) break;
@@ -994,14 +1003,27 @@ __global__ void __launch_bounds__(T_THREADS, 1) tc_tmem_kernel(const __grid_cons
       const uint32_t mrows = min((uint32_t)T_MROWS, jb.M - mb * T_MROWS);
       const uint32_t ncols = min((uint32_t)T_NCOLS, jb.d1 - nb * T_NCOLS);
       const uint64_t nstride = (uint64_t)2 * p.L * p.N;
-      for (uint32_t mm = 0; mm < mrows; ++mm) {
-        const uint32_t mg = mb * T_MROWS + mm, c = mg >> 1, rr = mg & 1;
-        const uint32_t sw = (mm & 7u) << 2;
-        uint32_t *orow = jb.out + (((uint64_t)c * jb.d1 + nb * T_NCOLS) * 2 + rr) * p.L * p.N + (uint64_t)l * p.N + t;
+      const uint64_t ln = (uint64_t)p.L * p.N;
+      uint32_t *to = jb.out + ((uint64_t)nb * T_NCOLS + lane) * nstride + (uint64_t)l * p.N + t;
+      for (uint32_t m0 = (uint32_t)(warp - W_STORE); m0 < mrows; m0 += NROW * NST) {
+        uint32_t v[NROW][T_NCOLS / 32];
 #pragma unroll
-        for (uint32_t hh = 0; hh < T_NCOLS / 32; ++hh) {
-          const uint32_t n = hh * 32 + lane;
-          if (n < ncols) orow[n * nstride] = out_stage[mm * T_NCOLS + (n ^ sw)];
+        for (uint32_t j = 0; j < NROW; ++j) {
+          const uint32_t mm = m0 + j * NST, sw = (mm & 7u) << 2;
+#pragma unroll
+          for (uint32_t hh = 0; hh < T_NCOLS / 32; ++hh)
+            asm volatile("ld.shared.u32 %0, [%1];"
+                         : "=r"(v[j][hh])
+                         : "r"(stage_s + 4 * (mm * T_NCOLS + ((hh * 32 + lane) ^ sw)))
+                         : "memory");
+        }
+#pragma unroll
+        for (uint32_t j = 0; j < NROW; ++j) {
+          const uint32_t mm = m0 + j * NST, mg = mb * T_MROWS + mm;
+          uint32_t *row = to + (uint64_t)(mg >> 1) * jb.d1 * nstride + (mg & 1u) * ln;
+#pragma unroll
+          for (uint32_t hh = 0; hh < T_NCOLS / 32; ++hh)
+            if (mm < mrows && hh * 32 + lane < ncols) row[hh * 32 * nstride] = v[j][hh];
         }
       }
       __syncwarp();
