@@ -258,10 +258,12 @@ class Clocks:
 KERNELS = {"rowsel_cc": (1, "rowsel_cc.cu", 1), "rowsel_imma": (2, "rowsel_imma.cu", 16),
            "tc_gemm": (4, "rowsel_tc.cu", 16), "tc_ingest": (4, "rowsel_tc.cu", 16),
            "tc_fused": (4, "rowsel_tc.cu", 16), "tc_cluster": (4, "rowsel_tc.cu", 16),
-           "tc_tmem": (4, "rowsel_tmem.cu", 12), "tc_tmem_pair": (4, "rowsel_tmem.cu", 12)}
-# tensor-core path variants that run the tensor-memory kernel (the variant
-# table in rowsel_tc.cu): 12 digit products per modular MAC, the others 16
-TMEM_VARIANT_IDS = (8, 9, 10, 11)
+           "tc_tmem": (4, "rowsel_tmem.cu", 12), "tc_tmem_pair": (4, "rowsel_tmem.cu", 12),
+           "tc_stream": (4, "rowsel_stream.cu", 12)}
+# tensor-core path variants that run the tensor-memory kernel or the streaming
+# kernel (the variant table in rowsel_tc.cu): 12 digit products per modular
+# MAC, the others 16
+TMEM_VARIANT_IDS = (8, 9, 10, 11, 12)
 
 
 def path_products(path, variant):

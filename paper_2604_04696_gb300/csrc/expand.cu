@@ -31,7 +31,7 @@
 //     time: 64 registers, 82 KB of shared memory at N = 4096, two CTAs per SM;
 //     Bound by instruction issue (2490 warp instructions a warp and node, 3440
 //     when each digit had its own transform and reduced after every round):
-//     32 clients, 274 outputs: 2.90 -> 1.99 ms;
+//     32 clients, 274 outputs: 2.90 -> 1.96 ms;
 //   - expand_split_kernel: for stages with few nodes, L digits CTAs per node
 //     (limb x digit), each repeating the inverse NTT and doing one digit.
 // The tree runs in place in the output array: stage j reads list[k], k < 2^j,
@@ -181,10 +181,11 @@ __global__ void __launch_bounds__(ntt::threads<LOGN>(), ntt::ctas_per_sm<LOGN>()
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
     fence_mbar_init();
-    if (p.bulk) {
-      mbar_arrive_expect_tx(&bar[0], 4 * N);
-      bulk_g2s(pa, expand_node<L, LOGN>(p, blockIdx.x / L).in + (size_t)h * N, 4 * N, &bar[0]);
-    }
+  }
+  wait_for_previous_stage();
+  if (b == 0 && p.bulk) {
+    mbar_arrive_expect_tx(&bar[0], 4 * N);
+    bulk_g2s(pa, expand_node<L, LOGN>(p, blockIdx.x / L).in + (size_t)h * N, 4 * N, &bar[0]);
   }
   __syncthreads();
   uint32_t ph = 0;
@@ -321,6 +322,7 @@ __global__ void __launch_bounds__(ntt::threads<LOGN>(), 1)
   }
   uint2 w[7];
   if (act) inv_first_twiddles<LOGN>(w, T, b);
+  wait_for_previous_stage();
   expand_load<L, LOGN>(p, node, h, stage, &bar);
 
   // 1. tau(a) on the owned slots of limb h, then its inverse NTT
@@ -418,13 +420,15 @@ int launch_stage(const ExpandParams &p, unsigned nodes, bool split, int dev, cud
   cfg.blockDim = dim3(ntt::threads<LOGN>());
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = cl;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = p.stage > 0 ? 2 : 1;   // stage 0 follows work that is not this call's
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, p);
   return e == cudaSuccess ? GPIR_OK : set_cuda_error(e);
 }

@@ -501,6 +501,22 @@ __device__ __forceinline__ void dcp_digits(const Ring &R, const Limb &T, uint32_
     d[i] = ((uint32_t)((int64_t)y >> (LOG_BASE * i)) & R.digit_mask[i]) + T.digit_add[i];
 }
 
+// Programmatic dependent launch: a stage's grid starts while the stage before
+// it finishes. It may read only what no earlier stage writes until it has
+// waited (the wait returns at once when the grid was launched without the
+// attribute), and it lets its own successor start only after that, so that what
+// a successor reads ahead was complete when this stage began.
+// Small stages are chains of barriers behind a launch, and the launch is what
+// this hides: one client's whole step 303 -> 283 us, ExpandQuery of 32 clients
+// 1.972 -> 1.956 ms.
+__device__ __forceinline__ void let_next_stage_start() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void wait_for_previous_stage() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  let_next_stage_start();
+}
+
 // Thread-block cluster helpers: the CTAs of a tree node hand each other
 // coefficient residues and partial sums through distributed shared memory.
 // They are pushed: the receiver reads its own shared memory after the barrier,
