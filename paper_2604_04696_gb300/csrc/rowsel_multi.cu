@@ -32,7 +32,8 @@ static int tc_jobs(const gpir_job_t *jobs, uint32_t njobs, cudaStream_t stream) 
     return GPIR_ENOMEM;
   }
   for (uint32_t k = 0; k < njobs; ++k)
-    part[pick_variant(jobs[k].db, jobs[k].batch, GPIR_PATH_TC) == kTcVariantStream].push_back(jobs[k]);
+    part[jobs[k].db->db_fields && pick_variant(jobs[k].db, jobs[k].batch, GPIR_PATH_TC) == kTcVariantStream].push_back(
+        jobs[k]);
   if (!part[1].empty()) {
     const int rc = rowsel_stream_launch(part[1].data(), (uint32_t)part[1].size(), stream);
     if (rc != GPIR_OK || part[0].empty()) return rc;

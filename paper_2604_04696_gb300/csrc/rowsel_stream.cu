@@ -669,25 +669,31 @@ PackStreamParams stream_shape(const gpir_db *db) {
 
 }  // namespace
 
-// The database tiles and column corrections of the streaming kernel.
+// The database tiles and column corrections of the streaming kernel. A database
+// that leaves no room for them is served by the other kernels.
 int rowsel_stream_prepare(gpir_db *db, cudaStream_t stream) {
   PackStreamParams pp = stream_shape(db);
   const uint64_t blocks = (uint64_t)pp.gpl * pp.L * pp.cblk * pp.kch;
   const size_t bytes = (size_t)blocks * pp.spg * S_TILE;
   const uint64_t slots = (uint64_t)pp.L * pp.N;
   const size_t corr_bytes = (size_t)slots * pp.cblk * S_COLS * 4;
-  if (blocks > 0x7fffffffull || (slots * pp.d1 + 255) / 256 > 0x7fffffffull) return GPIR_ETOOBIG;
+  if (blocks > 0x7fffffffull || (slots * pp.d1 + 255) / 256 > 0x7fffffffull) return GPIR_OK;
   cudaError_t e = dev_malloc(reinterpret_cast<void **>(&db->db_fields), bytes);
-  if (e != cudaSuccess) {
-    db->db_fields = nullptr;
-    return set_cuda_error(e);
+  if (e != cudaSuccess) db->db_fields = nullptr;
+  if (e == cudaSuccess) {
+    e = dev_malloc(reinterpret_cast<void **>(&db->db_corr), corr_bytes);
+    if (e != cudaSuccess) {
+      db->db_corr = nullptr;
+      cudaFree(db->db_fields);
+      db->db_fields = nullptr;
+    }
   }
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    return GPIR_OK;
+  }
+  if (e != cudaSuccess) return set_cuda_error(e);
   db->db_fields_bytes = bytes;
-  e = dev_malloc(reinterpret_cast<void **>(&db->db_corr), corr_bytes);
-  if (e != cudaSuccess) {
-    db->db_corr = nullptr;
-    return set_cuda_error(e);
-  }
   db->db_corr_bytes = corr_bytes;
   pp.tiles = db->db_fields;
   stream_pack_kernel<<<(unsigned)blocks, 256, 0, stream>>>(pp);

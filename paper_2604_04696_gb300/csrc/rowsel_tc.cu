@@ -2239,7 +2239,10 @@ int rowsel_tc_launch(const gpir_db *db, uint32_t batch, const uint32_t *ct, uint
     job.batch = batch;
     job.ct = ct;
     job.out = out;
-    return rowsel_stream_launch(&job, 1, stream);
+    const int rc = rowsel_stream_launch(&job, 1, stream);
+    if (rc != GPIR_ENOTSUP) return rc;
+    const FusedVariant &t = kFusedVariants[8];   // a database without its tiles
+    return tc_launch_tmem(db, batch, ct, out, (size_t)t.ring_mb << 20, t.lookahead_mb, t.hints, false, stream);
   }
   if (v.kind == kKindTmem || v.kind == kKindTmemPair) {
     const bool pr = v.kind == kKindTmemPair;

@@ -97,3 +97,38 @@ def test_several_jobs_in_one_launch(g):
     finally:
         for h in hs:
             h.close()
+
+
+@pytest.mark.parametrize("nth", [4, 5])
+def test_upload_without_room_for_its_tiles(g, nth):
+    """A database whose streaming tiles cannot be allocated (the fourth and
+    fifth allocation of an upload) is served by the other kernels, by itself,
+    in a multi-job call and where the streaming variant is asked for."""
+    import torch
+    from tests.gpu_util import to_dev, to_host
+    B, D0, D1, L, N = 4, 40, 24, 2, 2048
+    ct = synth.ct_tensor(77, B, D0, L, N, P28)
+    db = synth.db_tensor(77, D0, D1, L, N, P28)
+    want = oracle.rowsel(ct, db, list(P28))
+    params = g.gpir_params_create(N, list(P28))
+    h = None
+    try:
+        g.gpir_set_fail_alloc(nth)
+        h = g.gpir_db_upload(params, D0, D1, to_dev(db), True, 0)
+        assert g.gpir_set_fail_alloc(0) == 0
+        ctd, out = to_dev(ct), torch.empty((B, D1, 2, L, N), dtype=torch.int32, device="cuda")
+        for path in (g.GPIR_PATH_AUTO, g.GPIR_PATH_TC):
+            out.fill_(-1)
+            g.gpir_rowsel_batch(h, B, ctd, out, path)
+            g.gpir_sync(None, 20000)
+            assert np.array_equal(to_host(out), want)
+        g.gpir_set_variant(h, B, g.GPIR_PATH_TC, STREAM)
+        out.fill_(-1)
+        g.gpir_rowsel_multi([(h, B, ctd, out)], g.GPIR_PATH_TC)
+        g.gpir_sync(None, 20000)
+        assert np.array_equal(to_host(out), want)
+    finally:
+        g.gpir_set_fail_alloc(0)
+        if h is not None:
+            g.gpir_db_free(h)
+        g.gpir_params_destroy(params)
