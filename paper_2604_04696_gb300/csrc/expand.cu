@@ -502,11 +502,13 @@ extern "C" int gpir_expand_query(const gpir_params_t *params, uint32_t batch, ui
     p.ksub = (N >> st) + 1;
     const unsigned nodes = batch * p.nodes;
     // stage-aware choice (Sec. 4.4): the limb x digit split (which repeats the
-    // inverse NTT per digit) when its CTAs fit one per SM, the limb split
-    // otherwise. Measured at N = 4096, L = 2: the split is about 10% faster
-    // per stage up to 16 nodes and slower from 32 nodes up.
+    // inverse NTT per digit) when its clusters run at once, one CTA per SM, the
+    // limb split otherwise. A cluster's CTAs share a GPC, so not every SM can be
+    // used: 7/8 of them is below what fits. One stage at N = 4096, us, split /
+    // limb: 12.7 / 14.6 up to 16 nodes, 14.1 / 14.7 at 22 and 23, but 20.9 / 14.6
+    // at 24 and 25 (L = 2, 6 CTAs); 12.2 / 12.6 at 16 and equal at 30 to 38 (L = 1).
     const unsigned split_ctas = L * (L == 1 ? ntt::digits<1>() : ntt::digits<2>());
-    const bool split = (uint64_t)nodes * split_ctas <= (uint64_t)sm_count();
+    const bool split = (uint64_t)nodes * split_ctas * 8 <= (uint64_t)sm_count() * 7;
     const int tr = trace_begin(split ? "expand_stage_split" : "expand_stage", s);
     rc = L == 1 ? launch_stage_n<1>(p, nodes, split, dev, s) : launch_stage_n<2>(p, nodes, split, dev, s);
     trace_end(tr, s);
