@@ -559,6 +559,17 @@ __global__ void __launch_bounds__(S_THREADS, 1) tc_stream_kernel(const __grid_co
     const uint32_t u4 = lane >> 3, m = qw * 8 + (lane & 7);
     const int et = (int)threadIdx.x - 32 * SW_EPI0;
     const bool b0 = u4 & 1u, b1 = u4 >> 1;
+    // Barrier of the 8 warps: whether `v` held in all of them.
+    auto epi_all = [&](bool v) -> bool {
+      uint32_t r = v ? 1u : 0u;
+      asm volatile(
+          "{\n .reg .pred pin, pout;\n setp.ne.u32 pin, %1, 0;\n bar.red.and.pred pout, 1, %2, pin;\n"
+          " selp.u32 %0, 1, 0, pout;\n}"
+          : "=r"(r)
+          : "r"(r), "n"(32 * SN_EPI)
+          : "memory");
+      return r != 0;
+    };
     uint32_t *cell = stage + (8 * hf + u4) * S_COLS + (m ^ (u4 * 8));   // row 8 hf + u; + 4 rows: the same swizzle
     uint32_t grp = 0;
     bool ok = true;
@@ -603,9 +614,11 @@ __global__ void __launch_bounds__(S_THREADS, 1) tc_stream_kernel(const __grid_co
           }
         }
       }
-      if (!ok) break;
-      // the unit's 8 slots of every (row, column) leave together
-      asm volatile("bar.sync 1, %0;" ::"n"(32 * SN_EPI) : "memory");
+      // the unit's 8 slots of every (row, column) leave together. After an
+      // expired wait some of the 8 warps may still see their accumulator
+      // arrive and others not: they agree here, so that none is left waiting
+      // at the barrier below for a warp that has gone.
+      if (!epi_all(ok)) break;
       uint32_t v[2][8];
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
