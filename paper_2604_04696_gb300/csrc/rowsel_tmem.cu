@@ -80,7 +80,7 @@ constexpr int32_t kOffB = 512 * (1 + (1 << 10));
 
 // Warp roles (896 threads). Tensor-memory lane quarter of a warp = warp % 4.
 constexpr int W_PROD = 0, W_MMA = 1, W_STORE = 2;
-constexpr int W_RELAY = 3;                           // SM pair: hands finished groups to the odd CTA; else a second store warp
+constexpr int W_RELAY = 3;                           // SM pair: hands finished groups to the odd CTA; else the second store warp
 constexpr int W_CONV0 = 4, N_CONV = 8;               // two converter sets of 4 warps (quarters 0..3),
                                                      // set s converts stages s and s + 2
 constexpr int W_EPI0 = 12, N_EPI = 8;                // 8 epilogue warps: quarter, column half
@@ -160,6 +160,7 @@ struct TmemParams {
   uint32_t L, N, njobs, kch_max;
   uint32_t R, gpl, spg, lookahead;
   TmDiv R_d, gpl_d;
+  uint32_t store_warps;                 // warps that write outputs: 1 or 2
   uint32_t hints;                       // 1: raw boxes evict-first, ring stores evict-last in L2
   uint64_t n_entries, n_units, n_tasks; // over all jobs
   uint8_t *ring;                        // [R][8 slots][kch_max] x 8 KB
@@ -444,7 +445,7 @@ __global__ void __launch_bounds__(T_THREADS, 1) tc_tmem_kernel(const __grid_cons
     mbar_init(&box_bar[0], 1);
     mbar_init(&box_bar[1], 1);
     mbar_init(ostage_full, N_EPI);
-    mbar_init(ostage_empty, PAIR ? 1 : 2);
+    mbar_init(ostage_empty, PAIR ? 1 : p.store_warps);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -985,16 +986,18 @@ __global__ void __launch_bounds__(T_THREADS, 1) tc_tmem_kernel(const __grid_cons
         hb ^= 1u;
       }
     }
-  } else if (warp == W_STORE || (!PAIR && warp == W_RELAY)) {
-    // ---------------- output store warps (one in the pair form, else two) ----------------
-    // A store writes 32 words of 32 sectors. At few database rows (one group per
-    // unit) the output bounds the kernel: one warp, a load and a store in turn,
-    // was busy 83% of the time at 256 rows and 32 clients while the MMAs waited
-    // for accumulators. Two warps, and four rows read from the stage before any
-    // is written so that a warp's stores follow one another: 256x64, 2 limbs of
-    // 4096 slots, 32 clients 541 -> 501 us, 128 clients 2112 -> 1865 us.
-    constexpr uint32_t NST = PAIR ? 1 : 2, NROW = 4;
-    static_assert(T_MROWS % (NROW * NST) == 0, "whole steps of rows");
+  } else if (warp == W_STORE || (!PAIR && warp == W_RELAY && p.store_warps == 2)) {
+    // ---------------- output store warps (one in the pair form, else one or two) ----------------
+    // A store writes 32 words of 32 sectors. At few database rows the output
+    // bounds the kernel: one warp, a load and a store in turn, was busy 83% of
+    // the time at 256 rows and 32 clients while the MMAs waited for
+    // accumulators. Four rows are read from the stage before any is written, so
+    // that a warp's stores follow one another, and short units have a second
+    // warp (the rule stands at the launch): 256x64, 2 limbs of 4096 slots, 32
+    // clients 541 -> 508 us, 128 clients 2105 -> 1860 us.
+    constexpr uint32_t NROW = 4;
+    static_assert(T_MROWS % (NROW * 2) == 0, "whole steps of rows");
+    const uint32_t NST = PAIR ? 1u : p.store_warps;
     const uint32_t stage_s = smem_u32(out_stage);
     uint32_t ph = 0;
     for (;;) {
@@ -1429,6 +1432,14 @@ int tc_launch_tmem_jobs(const gpir_job_t *jobs, uint32_t njobs, size_t ring_targ
   e = cudaMemsetAsync(flags, 0, flag_bytes, stream);
   if (e != cudaSuccess) return set_cuda_error(e);
   tp.hints = hints;
+  // A second store warp where a unit has few k-chunks to hide its output behind.
+  // From 7 on one keeps up, and the second only takes issue slots from the
+  // others. One / two store warps, us (2 limbs of 4096 slots): 256x64, 32 clients
+  // 526 / 506; 320x100, 20 clients 869 / 797; 384x100, 20 clients 912 / 864; but
+  // 448x64, 32 clients 760 / 785; 512x64, 32 clients 832 / 886; 500x90, 50
+  // clients 2040 / 2084; 1024x128, 128 clients 7984 / 8164. Several jobs: by the
+  // longest one's units, which take most of the time.
+  tp.store_warps = pair || kch_max >= 7 ? 1 : 2;
   tp.lookahead =
       lookahead_mb == 0 ? 0u : (uint32_t)std::max<uint64_t>(2, ((uint64_t)lookahead_mb << 20) / entry_bytes);
   tp.err = device_error_word();
