@@ -222,9 +222,9 @@ long gpir_set_fail_alloc(long n);
  * shape (-1 if none chosen yet). Host-only. */
 int gpir_num_variants(int path);
 /* The path GPIR_PATH_AUTO resolves to for `batch` clients (tuned, else the
- * static rule when prepared: tensor cores from 8 clients up, and below that from
- * 2 clients on databases of more than 192 rows, from 5 on smaller ones, if the
- * database has enough 8-slot x 32-column tiles for the SMs). Host-only. */
+ * static rule when prepared: tensor cores from 8 clients up, and from 2 up where
+ * the database's rows, columns and slots fill the SMs well enough for the
+ * streaming kernel to be the faster one). Host-only. */
 int gpir_selected_path(const gpir_db_t *db, uint32_t batch);
 int gpir_selected_variant(const gpir_db_t *db, uint32_t batch, int path);
 /* Force a variant for (path, batch, D0, D1) of this database (testing). */

@@ -229,14 +229,10 @@ int pick_variant(const gpir_db *db, uint32_t batch, int path) {
 }
 
 // GPIR_PATH_AUTO: the path the autotuner measured fastest for this batch size,
-// else a static choice. Where the streaming kernel applies (up to 8 clients):
-// tensor cores from 2 clients on databases of more than 192 rows, from 5 on
-// smaller ones, whose units are too short to hide its pipeline's ends. N = 4096,
-// 2 limbs, us on the CUDA cores / streaming: 2 clients 211 / 131 and 3 clients
-// 213 / 132 (256x64), 4 clients 237 / 166 (600x8) and 244 / 202 (300x33), but 35 / 47
-// (64x32) and 49 / 55 (100x16); 8 clients 68 / 55 and 84 / 59 on those two; one
-// client 94 / 129 (256x64). Elsewhere: tensor cores from 8 clients (one client
-// wastes 15/16 of an MMA tile).
+// else a static choice: tensor cores from 8 clients on (a tile of 16 rows), and
+// for 2 to 7 where the streaming kernel beats the CUDA cores
+// (rowsel_stream_beats_cc). One client wastes 15/16 of an MMA tile: 94 us on the
+// CUDA cores, 129 streaming (256x64, N = 4096, 2 limbs).
 int resolve_path(const gpir_db *db, int path, uint32_t batch) {
   if (path == GPIR_PATH_AUTO) {
     {
@@ -245,8 +241,7 @@ int resolve_path(const gpir_db *db, int path, uint32_t batch) {
       if (it != db->variants->end()) return it->second;
     }
     const bool tc = db->path_mask & GPIR_PATH_TC, cc = db->path_mask & GPIR_PATH_CUDACORE;
-    const uint32_t from = !rowsel_stream_preferred(db, batch) ? 8u : db->d0 > 192 ? 2u : 5u;
-    if (tc && (batch >= from || !cc)) return GPIR_PATH_TC;
+    if (tc && (!cc || batch >= 8 || rowsel_stream_beats_cc(db, batch))) return GPIR_PATH_TC;
     if (cc) return GPIR_PATH_CUDACORE;
     if (db->path_mask & GPIR_PATH_IMMA) return GPIR_PATH_IMMA;
     return -1;

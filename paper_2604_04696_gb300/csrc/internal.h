@@ -143,6 +143,8 @@ int rowsel_stream_launch(const gpir_job_t *jobs, uint32_t njobs, cudaStream_t st
 constexpr int kTcVariantStream = 12;   // its tile variant
 // whether untuned batches of this database take it on the tensor-core path
 bool rowsel_stream_preferred(const gpir_db *db, uint32_t batch);
+// whether untuned batches of up to 7 clients take it rather than the CUDA cores
+bool rowsel_stream_beats_cc(const gpir_db *db, uint32_t batch);
 // The tensor-core workspace kept for (current device, stream), grown on demand
 // (never inside a stream capture: GPIR_ENOMEM then).
 int tc_stream_workspace(cudaStream_t stream, size_t need, uint8_t **out);

@@ -731,6 +731,30 @@ bool rowsel_stream_preferred(const gpir_db *db, uint32_t batch) {
   return (uint64_t)sh.gpl * sh.L * sh.cblk >= (uint64_t)sm_count();
 }
 
+// Untuned batches of 2 to 7 clients: the streaming kernel or the CUDA cores.
+// Both run one CTA per 8 slots x 32 columns of such a batch and take whole waves.
+// A streaming wave (one unit per SM) costs a fixed part, a part per step of 64
+// rows and a part per exact group of 256, all padded; a wave of the CUDA cores
+// (four CTAs per SM) costs its rows, twice as much from 5 clients on, which take
+// a tile of twice the height. In quarters of what a row costs the CUDA cores,
+// the streaming parts are 20, 30 and 60 at up to 4 clients and 20, 14 and 23 above:
+// fitted to 8,100 points (16 to 1025 rows, 1 to 300 columns, N = 128 to 8192, 1 to 4
+// limbs, 160 to 8192 units), where the choice is at most 7% behind the faster
+// kernel. us, CUDA cores / streaming: 5 clients 12.6 / 28.7 (16x48, N = 2048, 1
+// limb), 7 clients 39 / 92 (16x1, N = 4096, 4 limbs) and 387 / 222 (257x64, N =
+// 4096, 2 limbs); 3 clients 56 / 63 (257x33, N = 2048, 1 limb), but 56 / 33
+// (257x192, N = 256, 1 limb) and 217 / 200 (257x64, N = 4096, 2 limbs). Up to 192
+// rows batches of 2 to 4 clients stay on the CUDA cores.
+bool rowsel_stream_beats_cc(const gpir_db *db, uint32_t batch) {
+  if (batch < 2 || (batch < 5 && db->d0 <= 192) || !rowsel_stream_preferred(db, batch)) return false;
+  const PackStreamParams sh = stream_shape(db);
+  const uint64_t units = (uint64_t)sh.gpl * sh.L * sh.cblk, sms = (uint64_t)sm_count();
+  const uint64_t waves = (units + sms - 1) / sms, cc_waves = (units + 4 * sms - 1) / (4 * sms);
+  const uint64_t groups = (sh.kch + S_KGROUP - 1) / S_KGROUP;
+  const uint64_t cost = batch < 5 ? 20 + 30 * (uint64_t)sh.kch + 60 * groups : 20 + 14 * (uint64_t)sh.kch + 23 * groups;
+  return waves * cost <= 4 * cc_waves * db->d0;
+}
+
 // RowSel problems of one parameter set through the streaming kernel, at most
 // S_MAX_JOBS per launch. It needs no workspace.
 int rowsel_stream_launch(const gpir_job_t *jobs, uint32_t njobs, cudaStream_t stream) {
