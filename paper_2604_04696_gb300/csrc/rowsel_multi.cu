@@ -19,7 +19,9 @@ namespace gpir {
 // Tensor-core jobs of one call: one job runs the kernel tuned for its batch. Of
 // several, those whose variant is the streaming kernel run in its launches of 8
 // jobs, the others in one persistent tensor-memory launch per 8 jobs (databases
-// uploaded without its digit tiles: the two-pass kernels).
+// uploaded without its digit tiles: the two-pass kernels). The others go first:
+// they need a workspace, and a call that cannot have it has then launched none of
+// the streaming jobs.
 static int tc_jobs(const gpir_job_t *jobs, uint32_t njobs, cudaStream_t stream) {
   if (njobs == 1)
     return dispatch(jobs[0].db, jobs[0].batch, jobs[0].ct, jobs[0].out, GPIR_PATH_TC,
@@ -34,23 +36,27 @@ static int tc_jobs(const gpir_job_t *jobs, uint32_t njobs, cudaStream_t stream) 
   for (uint32_t k = 0; k < njobs; ++k)
     part[jobs[k].db->db_fields && pick_variant(jobs[k].db, jobs[k].batch, GPIR_PATH_TC) == kTcVariantStream].push_back(
         jobs[k]);
-  if (!part[1].empty()) {
-    const int rc = rowsel_stream_launch(part[1].data(), (uint32_t)part[1].size(), stream);
-    if (rc != GPIR_OK || part[0].empty()) return rc;
+  if (!part[0].empty()) {
+    bool tmem = true;
+    for (const gpir_job_t &j : part[0]) tmem = tmem && j.db->db_digits12 != nullptr;
+    const int rc = tmem ? rowsel_tmem_multi(part[0].data(), (uint32_t)part[0].size(), stream)
+                        : rowsel_tc_multi(part[0].data(), (uint32_t)part[0].size(), stream);
+    if (rc != GPIR_OK || part[1].empty()) return rc;
   }
-  bool tmem = true;
-  for (const gpir_job_t &j : part[0]) tmem = tmem && j.db->db_digits12 != nullptr;
-  return tmem ? rowsel_tmem_multi(part[0].data(), (uint32_t)part[0].size(), stream)
-              : rowsel_tc_multi(part[0].data(), (uint32_t)part[0].size(), stream);
+  return rowsel_stream_launch(part[1].data(), (uint32_t)part[1].size(), stream);
 }
 
 int rowsel_multi_launch(const gpir_job_t *jobs, uint32_t njobs, int path, cudaStream_t stream) {
   if (path == GPIR_PATH_AUTO) {
     // each job on the path gpir_rowsel_batch would take for it (small batches
-    // on the CUDA cores); the tensor-core jobs together
-    std::vector<gpir_job_t> tc;
-    try {
-      tc.reserve(njobs);   // push_back below then never allocates (no exception crosses the C ABI)
+    // on the CUDA cores); the tensor-core jobs together, and before the others,
+    // which need no workspace
+    std::vector<gpir_job_t> tc, rest;
+    std::vector<int> path_of;   // of the jobs in rest
+    try {   // push_back below then never allocates (no exception crosses the C ABI)
+      tc.reserve(njobs);
+      rest.reserve(njobs);
+      path_of.reserve(njobs);
     } catch (...) {
       return GPIR_ENOMEM;
     }
@@ -59,13 +65,16 @@ int rowsel_multi_launch(const gpir_job_t *jobs, uint32_t njobs, int path, cudaSt
       if (p < 0) return GPIR_ENOTSUP;
       if (p == GPIR_PATH_TC) {
         tc.push_back(jobs[k]);
-        continue;
+      } else {
+        rest.push_back(jobs[k]);
+        path_of.push_back(p);
       }
-      const int rc = dispatch(jobs[k].db, jobs[k].batch, jobs[k].ct, jobs[k].out, p,
-                              pick_variant(jobs[k].db, jobs[k].batch, p), stream);
-      if (rc) return rc;
     }
-    return tc.empty() ? GPIR_OK : tc_jobs(tc.data(), (uint32_t)tc.size(), stream);
+    int rc = tc.empty() ? GPIR_OK : tc_jobs(tc.data(), (uint32_t)tc.size(), stream);
+    for (size_t k = 0; k < rest.size() && rc == GPIR_OK; ++k)
+      rc = dispatch(rest[k].db, rest[k].batch, rest[k].ct, rest[k].out, path_of[k],
+                    pick_variant(rest[k].db, rest[k].batch, path_of[k]), stream);
+    return rc;
   }
   for (uint32_t k = 0; k < njobs; ++k)
     if (!(jobs[k].db->path_mask & path)) return GPIR_ENOTSUP;
