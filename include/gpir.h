@@ -93,7 +93,14 @@ int gpir_params_destroy(gpir_params_t *params);
  * against its limb's prime: GPIR_ERANGE if any is >= q_l. The database is
  * prepared once, before queries (the paper transposes its DB offline, Sec.
  * 5.2.1), so this call synchronizes `stream`. The caller keeps ownership of
- * `db_ntt`; the handle owns the device copies until gpir_db_free. */
+ * `db_ntt`; the handle owns the device copies until gpir_db_free.
+ * GPIR_PATH_TC holds 14 bytes per residue beside the 4 of the database (columns
+ * padded to 64, rows to 64), and where an eighth of the device's memory stays
+ * free then, a further 4 (columns padded to 32) with 4 per slot and column for
+ * the kernel that serves small batches. These are optional: when a later
+ * allocation of the library finds the device full they are freed, unless a
+ * captured launch refers to them, and small batches are served by the other
+ * kernels. */
 int gpir_db_upload(const gpir_params_t *params, uint32_t d0, uint32_t d1,
                    const uint32_t *db_ntt, int db_on_device, uint32_t path_mask,
                    void *stream, gpir_db_t **out);

@@ -47,7 +47,7 @@ static void fail_alloc_init() {
   g_fail_alloc.compare_exchange_strong(expect, n > 0 ? n : 0);
 }
 
-cudaError_t dev_malloc(void **p, size_t bytes) {
+cudaError_t dev_malloc(void **p, size_t bytes, bool optional) {
   fail_alloc_init();
   for (;;) {
     long v = g_fail_alloc.load();
@@ -60,7 +60,13 @@ cudaError_t dev_malloc(void **p, size_t bytes) {
       break;
     }
   }
-  return cudaMalloc(p, bytes);
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess) cudaGetLastError();   // reported here: the next launch's check must not find it
+  if (e == cudaErrorMemoryAllocation && !optional && rowsel_stream_give_back()) {
+    e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) cudaGetLastError();
+  }
+  return e;
 }
 
 unsigned int *device_error_word() {
@@ -394,8 +400,7 @@ int gpir_db_free(gpir_db_t *db) {
   if (db->db_pmajor) cudaFree(db->db_pmajor);
   if (db->db_digits) cudaFree(db->db_digits);
   if (db->db_digits12) cudaFree(db->db_digits12);
-  if (db->db_fields) cudaFree(db->db_fields);
-  if (db->db_corr) cudaFree(db->db_corr);
+  rowsel_stream_release(db);
   if (db->ws_ct) cudaFree(db->ws_ct);
   if (db->ws_out) cudaFree(db->ws_out);
   delete db->variants;
@@ -407,7 +412,7 @@ int gpir_db_free(gpir_db_t *db) {
 size_t gpir_db_device_bytes(const gpir_db_t *db) {
   if (!db) return 0;
   size_t b = (size_t)db->d0 * db->d1 * db->params.num_limbs * db->params.n * 4;
-  return b + db->db_digits_bytes + db->db_digits12_bytes + db->db_fields_bytes + db->db_corr_bytes;
+  return b + db->db_digits_bytes + db->db_digits12_bytes + rowsel_stream_bytes(db);
 }
 
 int gpir_rowsel_batch(const gpir_db_t *db, uint32_t batch, const uint32_t *ct_dev, uint32_t *out_dev, int path,

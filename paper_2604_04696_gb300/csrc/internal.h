@@ -57,8 +57,11 @@ struct gpir_db {
   // and the four 7-bit fields of the residues with the columns' corrections (rowsel_stream.cu).
   uint8_t *db_fields;
   size_t db_fields_bytes;
+  // They are given back when memory runs out, unless a captured launch refers to
+  // them (written and read as atomics; the others are guarded by the tiles' lock).
   uint32_t *db_corr;
   size_t db_corr_bytes;
+  mutable uint32_t tiles_captured;
   // Host-buffer entry point workspace.
   uint32_t *ws_ct, *ws_out;
   size_t ws_ct_bytes, ws_out_bytes;
@@ -75,7 +78,9 @@ int set_cuda_error(cudaError_t e);
 // Every device allocation of the library goes through this wrapper: cudaMalloc,
 // unless the allocation-failure injection (GPIR_FAIL_ALLOC /
 // gpir_set_fail_alloc) makes it fail with cudaErrorMemoryAllocation.
-cudaError_t dev_malloc(void **p, size_t bytes);
+// When the device is full the streaming tiles of the databases on it are given
+// back and the allocation is tried again, unless what is allocated is optional.
+cudaError_t dev_malloc(void **p, size_t bytes, bool optional = false);
 
 // TMA descriptor encoding (driver entry point resolved at first use).
 int encode_tiled_u32(CUtensorMap *map, const void *base, int rank, const uint64_t *dims,
@@ -140,6 +145,10 @@ int tc_launch_tmem(const gpir_db *db, uint32_t batch, const uint32_t *ct, uint32
 // launches of up to 8 jobs of one parameter set each.
 int rowsel_stream_prepare(gpir_db *db, cudaStream_t stream);
 int rowsel_stream_launch(const gpir_job_t *jobs, uint32_t njobs, cudaStream_t stream);
+bool rowsel_stream_has_tiles(const gpir_db *db);
+size_t rowsel_stream_bytes(const gpir_db *db);
+void rowsel_stream_release(gpir_db *db);   // at gpir_db_free
+bool rowsel_stream_give_back();            // frees the tiles on the current device; whether there were any
 constexpr int kTcVariantStream = 12;   // its tile variant
 // whether untuned batches of this database take it on the tensor-core path
 bool rowsel_stream_preferred(const gpir_db *db, uint32_t batch);

@@ -34,16 +34,20 @@ static int tc_jobs(const gpir_job_t *jobs, uint32_t njobs, cudaStream_t stream) 
     return GPIR_ENOMEM;
   }
   for (uint32_t k = 0; k < njobs; ++k)
-    part[jobs[k].db->db_fields && pick_variant(jobs[k].db, jobs[k].batch, GPIR_PATH_TC) == kTcVariantStream].push_back(
+    part[rowsel_stream_has_tiles(jobs[k].db) && pick_variant(jobs[k].db, jobs[k].batch, GPIR_PATH_TC) == kTcVariantStream].push_back(
         jobs[k]);
-  if (!part[0].empty()) {
+  const auto with_workspace = [&](const std::vector<gpir_job_t> &js) {
     bool tmem = true;
-    for (const gpir_job_t &j : part[0]) tmem = tmem && j.db->db_digits12 != nullptr;
-    const int rc = tmem ? rowsel_tmem_multi(part[0].data(), (uint32_t)part[0].size(), stream)
-                        : rowsel_tc_multi(part[0].data(), (uint32_t)part[0].size(), stream);
+    for (const gpir_job_t &j : js) tmem = tmem && j.db->db_digits12 != nullptr;
+    return tmem ? rowsel_tmem_multi(js.data(), (uint32_t)js.size(), stream)
+                : rowsel_tc_multi(js.data(), (uint32_t)js.size(), stream);
+  };
+  if (!part[0].empty()) {
+    const int rc = with_workspace(part[0]);
     if (rc != GPIR_OK || part[1].empty()) return rc;
   }
-  return rowsel_stream_launch(part[1].data(), (uint32_t)part[1].size(), stream);
+  const int rc = rowsel_stream_launch(part[1].data(), (uint32_t)part[1].size(), stream);
+  return rc == GPIR_ENOTSUP ? with_workspace(part[1]) : rc;   // tiles given back meanwhile
 }
 
 int rowsel_multi_launch(const gpir_job_t *jobs, uint32_t njobs, int path, cudaStream_t stream) {

@@ -70,6 +70,8 @@
 
 #include <algorithm>
 #include <mutex>
+#include <shared_mutex>
+#include <vector>
 
 #include "common.cuh"
 #include "tcgen05.cuh"
@@ -665,6 +667,20 @@ StLimb make_st_limb(uint32_t q) {
 std::mutex g_st_mu;
 bool g_st_attr_done[64];
 
+// The databases that hold tiles. A launch holds the lock shared until it is
+// enqueued; tiles are added, freed and given back with it held alone.
+std::shared_mutex g_tiles_mu;
+std::vector<gpir_db *> g_tiles;
+
+void free_tiles(gpir_db *db) {
+  uint8_t *fields = db->db_fields;
+  __atomic_store_n(&db->db_fields, (uint8_t *)nullptr, __ATOMIC_RELAXED);
+  if (fields) cudaFree(fields);
+  if (db->db_corr) cudaFree(db->db_corr);
+  db->db_corr = nullptr;
+  db->db_fields_bytes = db->db_corr_bytes = 0;
+}
+
 PackStreamParams stream_shape(const gpir_db *db) {
   PackStreamParams pp;
   memset(&pp, 0, sizeof(pp));
@@ -682,8 +698,45 @@ PackStreamParams stream_shape(const gpir_db *db) {
 
 }  // namespace
 
+bool rowsel_stream_has_tiles(const gpir_db *db) {
+  return __atomic_load_n(&db->db_fields, __ATOMIC_RELAXED) != nullptr;
+}
+
+size_t rowsel_stream_bytes(const gpir_db *db) {
+  std::shared_lock<std::shared_mutex> lk(g_tiles_mu);
+  return db->db_fields_bytes + db->db_corr_bytes;
+}
+
+void rowsel_stream_release(gpir_db *db) {
+  std::unique_lock<std::shared_mutex> lk(g_tiles_mu);
+  g_tiles.erase(std::remove(g_tiles.begin(), g_tiles.end(), db), g_tiles.end());
+  free_tiles(db);
+}
+
+// The tiles only make small batches faster, so no other allocation of the
+// library fails for them: when the device is full, those that no captured
+// launch refers to are freed (cudaFree synchronizes across all executing
+// streams, so the launches that read them are done), and their databases are
+// served by the other kernels from then on.
+bool rowsel_stream_give_back() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  std::unique_lock<std::shared_mutex> lk(g_tiles_mu);
+  const auto held = [&](const gpir_db *db) {
+    return db->device != dev || __atomic_load_n(&db->tiles_captured, __ATOMIC_RELAXED) != 0;
+  };
+  const auto keep = std::partition(g_tiles.begin(), g_tiles.end(), held);
+  if (keep == g_tiles.end()) return false;
+  for (auto it = keep; it != g_tiles.end(); ++it) free_tiles(*it);
+  g_tiles.erase(keep, g_tiles.end());
+  return true;
+}
+
 // The database tiles and column corrections of the streaming kernel. A database
-// that leaves no room for them is served by the other kernels.
+// that leaves no room for them is served by the other kernels: they are taken
+// only where an eighth of the device's memory stays free, for the caller's
+// buffers (128 clients' ciphertexts and outputs of a 4 GiB database are 10 GB of
+// a GB300's 35).
 int rowsel_stream_prepare(gpir_db *db, cudaStream_t stream) {
   PackStreamParams pp = stream_shape(db);
   const uint64_t blocks = (uint64_t)pp.gpl * pp.L * pp.cblk * pp.kch;
@@ -691,10 +744,14 @@ int rowsel_stream_prepare(gpir_db *db, cudaStream_t stream) {
   const uint64_t slots = (uint64_t)pp.L * pp.N;
   const size_t corr_bytes = (size_t)slots * pp.cblk * S_COLS * 4;
   if (blocks > 0x7fffffffull || (slots * pp.d1 + 255) / 256 > 0x7fffffffull) return GPIR_OK;
-  cudaError_t e = dev_malloc(reinterpret_cast<void **>(&db->db_fields), bytes);
+  size_t free_bytes = 0, total_bytes = 0;
+  cudaError_t e = cudaMemGetInfo(&free_bytes, &total_bytes);
+  if (e != cudaSuccess) return set_cuda_error(e);
+  if (free_bytes < bytes + corr_bytes + total_bytes / 8) return GPIR_OK;
+  e = dev_malloc(reinterpret_cast<void **>(&db->db_fields), bytes, true);
   if (e != cudaSuccess) db->db_fields = nullptr;
   if (e == cudaSuccess) {
-    e = dev_malloc(reinterpret_cast<void **>(&db->db_corr), corr_bytes);
+    e = dev_malloc(reinterpret_cast<void **>(&db->db_corr), corr_bytes, true);
     if (e != cudaSuccess) {
       db->db_corr = nullptr;
       cudaFree(db->db_fields);
@@ -716,7 +773,14 @@ int rowsel_stream_prepare(gpir_db *db, cudaStream_t stream) {
   e = cudaGetLastError();
   if (e != cudaSuccess) return set_cuda_error(e);
   e = cudaStreamSynchronize(stream);
-  return e == cudaSuccess ? GPIR_OK : set_cuda_error(e);
+  if (e != cudaSuccess) return set_cuda_error(e);
+  std::unique_lock<std::shared_mutex> lk(g_tiles_mu);
+  try {
+    g_tiles.push_back(db);
+  } catch (...) {   // no exception crosses the C ABI
+    free_tiles(db);
+  }
+  return GPIR_OK;
 }
 
 // Untuned batches take the streaming kernel when they are one block of 16 rows
@@ -726,7 +790,7 @@ int rowsel_stream_prepare(gpir_db *db, cudaStream_t stream) {
 // of rows the database is converted twice and the gain is gone: 16 clients
 // 284 / 277 (256x64), 1375 / 1965 (1024x128).
 bool rowsel_stream_preferred(const gpir_db *db, uint32_t batch) {
-  if (!db->db_fields || batch > S_ROWS / 2) return false;
+  if (batch > S_ROWS / 2 || !rowsel_stream_has_tiles(db)) return false;
   const PackStreamParams sh = stream_shape(db);
   return (uint64_t)sh.gpl * sh.L * sh.cblk >= (uint64_t)sm_count();
 }
@@ -758,10 +822,15 @@ bool rowsel_stream_beats_cc(const gpir_db *db, uint32_t batch) {
 // RowSel problems of one parameter set through the streaming kernel, at most
 // S_MAX_JOBS per launch. It needs no workspace.
 int rowsel_stream_launch(const gpir_job_t *jobs, uint32_t njobs, cudaStream_t stream) {
+  std::shared_lock<std::shared_mutex> lk_tiles(g_tiles_mu);
   for (uint32_t k = 0; k < njobs; ++k)
     if (!jobs[k].db->db_fields || !jobs[k].db->db_corr) return GPIR_ENOTSUP;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(stream, &cs);
+  if (e != cudaSuccess || cs != cudaStreamCaptureStatusNone)   // its replays will read these tiles
+    for (uint32_t k = 0; k < njobs; ++k) __atomic_store_n(&jobs[k].db->tiles_captured, 1u, __ATOMIC_RELAXED);
   int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return set_cuda_error(e);
   if (dev < 0 || dev >= 64) return GPIR_EINVAL;
   {
