@@ -216,6 +216,7 @@ __global__ void __launch_bounds__(ntt::threads<LOGN>(), ntt::ctas_per_sm<LOGN>()
         src = (src + step) & (N - 1);
       }
     }
+    // (no barrier since the previous node's transform: it read what this thread writes first)
     inverse<LOGN>(a, work, w, T, b, act);
     if (b == 0 && p.bulk) {
       // every thread has read a, and the previous node's b, before the barriers of the transform

@@ -393,7 +393,11 @@ __device__ __forceinline__ void inv_middles(uint32_t *buf, uint2 (&w)[7], const 
 // slot b + (N/8) e, values in [0, 16q) (lazy: congruent mod q, not reduced).
 // Every thread of the CTA must call it (it holds __syncthreads); act = b < N/8.
 // Before its first barrier a thread writes only the positions b + (N/8) k of
-// the buffers. They are free again once the next barrier of the CTA has passed.
+// the buffers; after its last one it reads only the positions 8 brv(b) + k.
+// Those are also the positions that inverse() writes before its first barrier,
+// in the same thread, so an inverse() may follow with no barrier in between
+// (ExpandQuery's loop over nodes with one limb); any other use of the buffers
+// waits for the next barrier of the CTA.
 template <int LOGN, int P>
 __device__ __forceinline__ void forward(uint32_t (&v)[P][8], uint32_t *const (&buf)[P], const Limb &T, uint32_t b,
                                         bool act) {
@@ -448,8 +452,9 @@ __device__ __forceinline__ void inv_first_twiddles(uint2 (&w)[7], const Limb &T,
 
 // Inverse NTT of one polynomial of one limb. In: v[e] = slot b + (N/8) e,
 // values < 2q, and w from inv_first_twiddles. Out: v[k] = coefficient
-// b + (N/8) k, below q. After its last barrier a thread reads only the
-// positions b + (N/8) k of the buffer.
+// b + (N/8) k, below q. Before its first barrier a thread writes only the
+// positions 8 brv(b) + k of the buffer; after its last one it reads only the
+// positions b + (N/8) k.
 template <int LOGN>
 __device__ __forceinline__ void inverse(uint32_t (&v)[1][8], uint32_t *buf, uint2 (&w)[7], const Limb &T,
                                         uint32_t b, bool act) {
