@@ -56,6 +56,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "tcgen05.cuh"
@@ -701,14 +702,6 @@ __global__ void __launch_bounds__(T_THREADS, 1) tc_tmem_kernel(const __grid_cons
         }
         break;
       }
-      // this ring tile is in shared memory. Copies complete in any order, so
-      // the unit's last landing does not tell that the others have read their
-      // part of the entry; but a set waits for its own k-chunks in order, so
-      // at the set's last one all of its copies have. One count per set and
-      // unit: with one per k-chunk the division and the atomic cost 3% at 1024
-      // rows (128 columns: 16 clients 1.405 -> 1.363 ms, 128 clients 8.30 -> 8.03 ms).
-      if (qw == 0 && lane == 0 && (tag >> 32))
-        atomicAdd(&p.consumed[entry_of((uint32_t)tag)], (uint32_t)(tag >> 32));
       // this thread's digit plane: 8 bytes per k octet (conflict-free: the
       // warp's 32 reads of a step cover every bank twice)
       const uint2 *row = reinterpret_cast<const uint2 *>(rslots + r * T_RAW_TILE) + m * 32;
@@ -721,6 +714,14 @@ __global__ void __launch_bounds__(T_THREADS, 1) tc_tmem_kernel(const __grid_cons
         wv[4 * j + 2] = plane_pair(z.y, 0x5140u);
         wv[4 * j + 3] = plane_pair(z.y, 0x5342u);
       }
+      // The ring tile has landed. Copies complete in any order, so the unit's
+      // last landing does not tell that the others have read their part of the
+      // entry; but a set waits for its own k-chunks in order, so at the set's
+      // last one all of its copies have. One count per set and unit: with one
+      // per k-chunk the division and the atomic cost 3% at 1024 rows (128
+      // columns: 16 clients 1.405 -> 1.363 ms, 128 clients 8.30 -> 8.03 ms).
+      if (qw == 0 && lane == 0 && (tag >> 32))
+        atomicAdd(&p.consumed[entry_of((uint32_t)tag)], (uint32_t)(tag >> 32));
       const uint64_t tst = PROF ? clock64() : 0;
       if (conv_counter) pc[PROF ? kTCBusy : 0] += tst - tconv;
       // the A buffer's previous k-chunk must have been read by its MMAs before
@@ -991,13 +992,14 @@ __global__ void __launch_bounds__(T_THREADS, 1) tc_tmem_kernel(const __grid_cons
     // A store writes 32 words of 32 sectors. At few database rows the output
     // bounds the kernel: one warp, a load and a store in turn, was busy 83% of
     // the time at 256 rows and 32 clients while the MMAs waited for
-    // accumulators. Four rows are read from the stage before any is written, so
-    // that a warp's stores follow one another, and short units have a second
-    // warp (the rule stands at the launch): 256x64, 2 limbs of 4096 slots, 32
-    // clients 541 -> 508 us, 128 clients 2105 -> 1860 us.
-    constexpr uint32_t NROW = 4;
+    // accumulators. Short units have two warps (the rule stands at the launch),
+    // each reading two rows of the stage before it writes them, so that its
+    // stores follow one another (2 limbs of 4096 slots, 256x64, 32 clients: 541 ->
+    // 506 us; four rows at a time 3% slower at one k-chunk). Long units hide
+    // their output behind the MMAs, and one warp, row by row, disturbs those
+    // less (500x121, 128 clients: 4.28 -> 4.18 ms).
+    constexpr uint32_t NROW = PAIR ? 4 : 2;
     static_assert(T_MROWS % (NROW * 2) == 0, "whole steps of rows");
-    const uint32_t NST = PAIR ? 1u : p.store_warps;
     const uint32_t stage_s = smem_u32(out_stage);
     uint32_t ph = 0;
     for (;;) {
@@ -1014,25 +1016,41 @@ __global__ void __launch_bounds__(T_THREADS, 1) tc_tmem_kernel(const __grid_cons
       const uint64_t nstride = (uint64_t)2 * p.L * p.N;
       const uint64_t ln = (uint64_t)p.L * p.N;
       uint32_t *to = jb.out + ((uint64_t)nb * T_NCOLS + lane) * nstride + (uint64_t)l * p.N + t;
-      for (uint32_t m0 = (uint32_t)(warp - W_STORE); m0 < mrows; m0 += NROW * NST) {
-        uint32_t v[NROW][T_NCOLS / 32];
+      const auto store_rows = [&](auto nst) {
+        constexpr uint32_t NST = decltype(nst)::value;
+        for (uint32_t m0 = (uint32_t)(warp - W_STORE); m0 < mrows; m0 += NROW * NST) {
+          uint32_t v[NROW][T_NCOLS / 32];
 #pragma unroll
-        for (uint32_t j = 0; j < NROW; ++j) {
-          const uint32_t mm = m0 + j * NST, sw = (mm & 7u) << 2;
+          for (uint32_t j = 0; j < NROW; ++j) {
+            const uint32_t mm = m0 + j * NST, sw = (mm & 7u) << 2;
 #pragma unroll
-          for (uint32_t hh = 0; hh < T_NCOLS / 32; ++hh)
-            asm volatile("ld.shared.u32 %0, [%1];"
-                         : "=r"(v[j][hh])
-                         : "r"(stage_s + 4 * (mm * T_NCOLS + ((hh * 32 + lane) ^ sw)))
-                         : "memory");
+            for (uint32_t hh = 0; hh < T_NCOLS / 32; ++hh)
+              asm volatile("ld.shared.u32 %0, [%1];"
+                           : "=r"(v[j][hh])
+                           : "r"(stage_s + 4 * (mm * T_NCOLS + ((hh * 32 + lane) ^ sw)))
+                           : "memory");
+          }
+#pragma unroll
+          for (uint32_t j = 0; j < NROW; ++j) {
+            const uint32_t mm = m0 + j * NST, mg = mb * T_MROWS + mm;
+            uint32_t *row = to + (uint64_t)(mg >> 1) * jb.d1 * nstride + (mg & 1u) * ln;
+#pragma unroll
+            for (uint32_t hh = 0; hh < T_NCOLS / 32; ++hh)
+              if (mm < mrows && hh * 32 + lane < ncols) row[hh * 32 * nstride] = v[j][hh];
+          }
         }
-#pragma unroll
-        for (uint32_t j = 0; j < NROW; ++j) {
-          const uint32_t mm = m0 + j * NST, mg = mb * T_MROWS + mm;
+      };
+      if (PAIR) {
+        store_rows(std::integral_constant<uint32_t, 1>());
+      } else if (p.store_warps == 2) {
+        store_rows(std::integral_constant<uint32_t, 2>());
+      } else {
+        for (uint32_t mm = 0; mm < mrows; ++mm) {
+          const uint32_t mg = mb * T_MROWS + mm, sw = (mm & 7u) << 2;
           uint32_t *row = to + (uint64_t)(mg >> 1) * jb.d1 * nstride + (mg & 1u) * ln;
 #pragma unroll
           for (uint32_t hh = 0; hh < T_NCOLS / 32; ++hh)
-            if (mm < mrows && hh * 32 + lane < ncols) row[hh * 32 * nstride] = v[j][hh];
+            if (hh * 32 + lane < ncols) row[hh * 32 * nstride] = out_stage[mm * T_NCOLS + ((hh * 32 + lane) ^ sw)];
         }
       }
       __syncwarp();
@@ -1366,6 +1384,7 @@ int tc_launch_tmem_jobs(const gpir_job_t *jobs, uint32_t njobs, size_t ring_targ
   tp.gpl = (N + 7) / 8;
   tp.spg = N < 8 ? N : 8u;
   uint64_t entries = 0, units = 0, tasks = 0;
+  uint64_t long_work = 0, short_work = 0;   // k-chunks of the jobs with 7 and more of them a unit, and of the others
   uint32_t kch_max = 1;
   for (uint32_t k = 0; k < njobs; ++k) {
     const gpir_db *db = jobs[k].db;
@@ -1388,7 +1407,9 @@ int tc_launch_tmem_jobs(const gpir_job_t *jobs, uint32_t njobs, size_t ring_targ
     jb.out = jobs[k].out;
     const uint64_t ne = (uint64_t)tp.gpl * L * jb.mblk;
     entries += ne;
-    units += (pair ? ne / 2 : ne) * jb.upe;
+    const uint64_t nu = (pair ? ne / 2 : ne) * jb.upe;
+    units += nu;
+    (jb.kch >= 7 ? long_work : short_work) += nu * jb.kch;
     tasks += ne * jb.kch;
     kch_max = std::max(kch_max, jb.kch);
     const uint64_t dims[5] = {N, L, 2, db->d0, jobs[k].batch};
@@ -1432,14 +1453,13 @@ int tc_launch_tmem_jobs(const gpir_job_t *jobs, uint32_t njobs, size_t ring_targ
   e = cudaMemsetAsync(flags, 0, flag_bytes, stream);
   if (e != cudaSuccess) return set_cuda_error(e);
   tp.hints = hints;
-  // A second store warp where a unit has few k-chunks to hide its output behind.
-  // From 7 on one keeps up, and the second only takes issue slots from the
-  // others. One / two store warps, us (2 limbs of 4096 slots): 256x64, 32 clients
-  // 526 / 506; 320x100, 20 clients 869 / 797; 384x100, 20 clients 912 / 864; but
-  // 448x64, 32 clients 760 / 785; 512x64, 32 clients 832 / 886; 500x90, 50
-  // clients 2040 / 2084; 1024x128, 128 clients 7984 / 8164. Several jobs: by the
-  // longest one's units, which take most of the time.
-  tp.store_warps = pair || kch_max >= 7 ? 1 : 2;
+  // A second store warp where a unit has few k-chunks to hide its output behind:
+  // below 7. One / two store warps against one earlier form of both, the mean of
+  // 16 to 128 clients (2 limbs of 4096 slots): 256x121 1.05 / 0.96, 384x121 1.01 /
+  // 0.99, but 420x64 0.96 / 1.00, 420x121 0.99 / 1.00, 500x64 0.95 / 1.01, 500x121 0.98 /
+  // 1.00, 1024x128 0.96 / 0.97. Several jobs: one where the long ones have most of
+  // the work (a short job loses up to 10%, a long one gains 3%).
+  tp.store_warps = pair || long_work >= 2 * short_work ? 1 : 2;
   tp.lookahead =
       lookahead_mb == 0 ? 0u : (uint32_t)std::max<uint64_t>(2, ((uint64_t)lookahead_mb << 20) / entry_bytes);
   tp.err = device_error_word();
