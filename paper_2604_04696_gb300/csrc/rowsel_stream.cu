@@ -315,7 +315,8 @@ __global__ void __launch_bounds__(S_THREADS, 1) tc_stream_kernel(const __grid_co
   uint64_t *acc_empty = acc_full + S_SLOTS;                   // [8] drained
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + S_SLOTS);
   volatile uint32_t *abort_flag = tmem_slot + 1;
-  static_assert(8 * (2 * S_RING + 8 + 2 * S_ABUF + 2 * S_SLOTS + 1) <= 1024, "barrier area exceeds its reservation");
+  volatile uint32_t *epi_failed = tmem_slot + 2;             // an epilogue warp's wait has expired
+  static_assert(8 * (2 * S_RING + 8 + 2 * S_ABUF + 2 * S_SLOTS + 2) <= 1024, "barrier area exceeds its reservation");
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -338,6 +339,7 @@ __global__ void __launch_bounds__(S_THREADS, 1) tc_stream_kernel(const __grid_co
       mbar_init(&acc_empty[i], SN_EPI);
     }
     *abort_flag = 0;
+    *epi_failed = 0;
     fence_mbar_init();
   }
   if (warp == SW_MMA0) {
@@ -561,17 +563,6 @@ __global__ void __launch_bounds__(S_THREADS, 1) tc_stream_kernel(const __grid_co
     const uint32_t u4 = lane >> 3, m = qw * 8 + (lane & 7);
     const int et = (int)threadIdx.x - 32 * SW_EPI0;
     const bool b0 = u4 & 1u, b1 = u4 >> 1;
-    // Barrier of the 8 warps: whether `v` held in all of them.
-    auto epi_all = [&](bool v) -> bool {
-      uint32_t r = v ? 1u : 0u;
-      asm volatile(
-          "{\n .reg .pred pin, pout;\n setp.ne.u32 pin, %1, 0;\n bar.red.and.pred pout, 1, %2, pin;\n"
-          " selp.u32 %0, 1, 0, pout;\n}"
-          : "=r"(r)
-          : "r"(r), "n"(32 * SN_EPI)
-          : "memory");
-      return r != 0;
-    };
     uint32_t *cell = stage + (8 * hf + u4) * S_COLS + (m ^ (u4 * 8));   // row 8 hf + u; + 4 rows: the same swizzle
     uint32_t grp = 0;
     bool ok = true;
@@ -618,9 +609,12 @@ __global__ void __launch_bounds__(S_THREADS, 1) tc_stream_kernel(const __grid_co
       }
       // the unit's 8 slots of every (row, column) leave together. After an
       // expired wait some of the 8 warps may still see their accumulator
-      // arrive and others not: they agree here, so that none is left waiting
-      // at the barrier below for a warp that has gone.
-      if (!epi_all(ok)) break;
+      // arrive and others not: they agree here, by a word written before the
+      // barrier only, so that none is left waiting at the next one for a warp
+      // that has gone.
+      if (!ok) *epi_failed = 1;
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * SN_EPI) : "memory");
+      if (*epi_failed) break;
       uint32_t v[2][8];
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
