@@ -29,9 +29,11 @@
 //     forward transform together (see ntt.cuh), and the multiply-accumulate
 //     starts when they are done, so its 64-bit sums live for one slot at a
 //     time: 64 registers, 82 KB of shared memory at N = 4096, two CTAs per SM;
-//     Bound by instruction issue (2490 warp instructions a warp and node, 3440
-//     when each digit had its own transform and reduced after every round):
-//     32 clients, 274 outputs: 2.90 -> 1.96 ms;
+//     2420 warp instructions a warp and node (3440 when each digit had its own
+//     transform and reduced after every round): 32 clients, 274 outputs: 2.90 ->
+//     1.96 ms. No pipe is full (issue slots 51% busy, ALU 37%, FMA 21%): between
+//     the CTA-wide barriers of a transform's rounds the warps wait for each
+//     other, for key rows and for the multiply pipe;
 //   - expand_split_kernel: for stages with few nodes, L digits CTAs per node
 //     (limb x digit), each repeating the inverse NTT and doing one digit.
 // The tree runs in place in the output array: stage j reads list[k], k < 2^j,

@@ -39,7 +39,7 @@
 // unit:
 //   - warp 0 copies the 8 slots' database tiles (8 KB each, contiguous in the
 //     packed layout) into a ring of shared-memory slots;
-//   - warp 2 loads the raw boxes, 4 clients each; boxes past the batch are left
+//   - warp 1 loads the raw boxes, 4 clients each; boxes past the batch are left
 //     out (their rows' products are never stored);
 //   - 8 ingest warps split the residues into fp16 digits and write the 8
 //     slots' operand tiles (48 rows v*16 + m, 64 k, 128-byte swizzle);
@@ -61,7 +61,7 @@
 // time, and the chains between them (convert, issue, commit, drain) set the pace
 // (256x64, 2 limbs: 8 clients 237 -> 154 us against the tensor-memory kernel, 67%
 // of the copy rate; 3 clients 213 -> 132 us against the CUDA cores; 3 clients on
-// 1024x128 1494 -> 894 us). Tried: four MMA warps (156 us), waits that suspend the
+// 1024x128 1494 -> 898 us). Tried: four MMA warps (156 us), waits that suspend the
 // warp (157 us), reads through generic pointers (179 us).
 #include <cuda.h>
 #include <cuda_fp16.h>

@@ -749,8 +749,8 @@ __global__ void __launch_bounds__(T_THREADS, 1) tc_tmem_kernel(const __grid_cons
     // ---------------- MMA issuer ----------------
     // The warp stays converged and one elected lane issues: from a lone thread
     // of a diverged warp four MMAs and their commits took half again as long
-    // (618 against 472 cycles a k-chunk in a stand-alone loop; here 4 GiB, 128
-    // clients: 7.86 -> 7.58 ms).
+    // (618 against 472 cycles a k-chunk in a stand-alone loop; here 1024x128, 128
+    // clients, both builds in turn on one GPU: 8.45 -> 8.29 ms).
     uint32_t leader;
     asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(leader));
     // k-chunk i of this CTA sits in part i % KPB of A buffer (i / KPB) %
